@@ -41,8 +41,7 @@ __global__ void __launch_bounds__(BATCH_BT, 65536 / (BATCH_BT * 128))
     k_batch_step(const RunDesc* __restrict__ runs, const int2* __restrict__ tasks, int4 phase_end, long long T,
                  BatchCtrl* bc, unsigned long long* done, int R, long long spin_limit, int tune)
 {
-    __shared__ float4 sj[BATCH_BT];
-    __shared__ float s_acc[2][3][BATCH_BT / 32][SYM_SUB];
+    __shared__ SymShared<BATCH_BT / 32, BATCH_BT * IPT> sym;
     __shared__ long long s_task;
     __shared__ int s_timeout;
     const unsigned long long bstep = bc->step;
@@ -86,9 +85,9 @@ __global__ void __launch_bounds__(BATCH_BT, 65536 / (BATCH_BT * 128))
             if (d.F.sym) {
                 int I, J;
                 tri_unit(tk.y, d.F.JS, I, J);
-                sym2_unit<BATCH_BT, IPT>(d.B.fpos, d.F, I, J, s_acc, sj);
+                sym2_unit<BATCH_BT, IPT>(d.B.fpos, d.F, I, J, sym);
             } else {
-                forces_unit<BATCH_BT, IPT>(d.B.fpos, d.B.part, d.F, tk.y / d.F.JS, tk.y % d.F.JS, sj);
+                forces_unit<BATCH_BT, IPT>(d.B.fpos, d.B.part, d.F, tk.y / d.F.JS, tk.y % d.F.JS, sym.sj);
             }
             break;
         case 2: kick_body<BATCH_BT, 1>(d.P, d.B, d.F, tune ? 1 : 0, tk.y); break;

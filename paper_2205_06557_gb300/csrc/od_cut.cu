@@ -263,8 +263,7 @@ __global__ void __launch_bounds__(BT, (IPT == 8 ? 65536 / (BT * 128) : 1))
     k_forces_cut(const float4* __restrict__ fsort, ForceArgs F, const int2* __restrict__ units,
                  const int* __restrict__ n_units)
 {
-    __shared__ float s_acc[2][3][BT / 32][SYM_SUB];
-    __shared__ float4 sj[BT];
+    __shared__ SymShared<BT / 32, BT * IPT> S;
     __shared__ long long s_u;
     const long long U = *n_units;
     for (;;) {
@@ -272,9 +271,9 @@ __global__ void __launch_bounds__(BT, (IPT == 8 ? 65536 / (BT * 128) : 1))
         if (u >= U) break;
         const int2 t = units[u];  // (I, J | plain flag)
         if (t.y & CUT_PLAIN)
-            sym2_unit<BT, IPT, false>(fsort, F, t.x, t.y & (CUT_PLAIN - 1), s_acc, sj);
+            sym2_unit<BT, IPT, false>(fsort, F, t.x, t.y & (CUT_PLAIN - 1), S);
         else
-            sym2_unit<BT, IPT, true>(fsort, F, t.x, t.y, s_acc, sj);
+            sym2_unit<BT, IPT, true>(fsort, F, t.x, t.y, S);
     }
     leave_queue(F.sched);
 }

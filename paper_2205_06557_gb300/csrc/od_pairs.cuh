@@ -342,25 +342,105 @@ __device__ __forceinline__ f32x2 pair_c3x2_cut(f32x2 dx, f32x2 dy, f32x2 dz, flo
     return mul2(mul2(e, mul2(ri, ri)), switch_bracket2(s, ri, s0, w_inv));
 }
 
-constexpr int SYM_SUB = 128;  // sources per combine step of the symmetric kernels
+// ------------------------------------------- symmetric units on packed FP32 pairs
+// One warp's part of a symmetric unit: a group of SYM_GRP = 64 sources against 32 IPT
+// targets (IPT per lane).  The group's positions are staged in the warp's shared memory as 32
+// packets (ions j and j + 32), each stored twice, so that at rotation r lane l reads packet
+// (l + r) & 31 at the fixed offset l + r: after 32 rotations every lane has met every source.
+// The packet's accumulator travels with it, one lane per rotation by shuffles, and is back on
+// lane (packet index) after the last.  Every FP32 operation of the pair term acts on the
+// packet's two sources in one f32x2 instruction.
+//
+// What bounds it: the FP32 pipe (17 operations per unordered pair) and the register file
+// behind it.  An f32x2 FMA with three different 64-bit operands issues every ~3.6 cycles
+// per scheduler instead of 2 (add, mul and FMA with a repeated operand: 2.2-2.8), and six of
+// the 17 are such FMAs.  Reading the travelling positions from shared memory instead of
+// shuffling them takes six of the twelve shuffles of a rotation, and their dependence on
+// the previous rotation, out of the loop.  k_forces_sym2<64,8>, 122,880 ions, 2070 MHz: 4.30 ms
+// (73% of the FP32 pipe's pair rate) with shuffled positions, two rotations per loop step and
+// 16 warps per SM at 128 registers; 4.22 ms with staged positions; 4.13 ms with 12 warps at 168
+// registers; 4.03 ms (79%) with four rotations per step and the sources' sums first.  Every sum
+// is made in the same order in all of them (the same bits).  Also measured: scalar
+// accumulations of the packed coefficients (twice the issue slots) 4.3-4.8 ms, 4 or 6 targets
+// per lane 4.3-4.4 ms.
+constexpr int SYM_GRP = 64;
+
+struct WarpStage {
+    f32x2 x[64], y[64], z[64];
+};
+
+// Sources pa (ion `lane` of the group) and pb (ion 32 + lane).  BOTH: the sources' sums go to b
+// (x, y, z of ion `lane`, then of ion 32 + lane) with the target-side sign; otherwise (a group
+// of the targets' own tile: each ordered pair met once) only the targets' sums are made, and
+// a self pair (d = 0) adds nothing.  CUT: the switched coefficient.
+template <int IPT, bool CUT, bool BOTH>
+__device__ __forceinline__ void sym2_group(float4 pa, float4 pb, const float (&xi)[IPT], const float (&yi)[IPT],
+                                           const float (&zi)[IPT], f32x2 (&ax)[IPT], f32x2 (&ay)[IPT],
+                                           f32x2 (&az)[IPT], float (&b)[6], WarpStage& S, float s0, float w_inv)
+{
+    const int lane = threadIdx.x & 31, src = (lane + 1) & 31;
+    __syncwarp();  // the previous group's reads are done
+    S.x[lane] = S.x[32 + lane] = pk2(pa.x, pb.x);
+    S.y[lane] = S.y[32 + lane] = pk2(pa.y, pb.y);
+    S.z[lane] = S.z[32 + lane] = pk2(pa.z, pb.z);
+    __syncwarp();
+    f32x2 bx = 0ull, by = 0ull, bz = 0ull;
+#pragma unroll 4
+    for (int r = 0; r < 32; ++r) {
+        const f32x2 xj = S.x[lane + r], yj = S.y[lane + r], zj = S.z[lane + r];
+#pragma unroll
+        for (int k = 0; k < IPT; ++k) {
+            const f32x2 dx = sub2(xj, pk2(xi[k], xi[k])), dy = sub2(yj, pk2(yi[k], yi[k])),
+                        dz = sub2(zj, pk2(zi[k], zi[k]));
+            const f32x2 c3 = CUT ? pair_c3x2_cut(dx, dy, dz, s0, w_inv) : pair_c3x2(dx, dy, dz);
+            if (BOTH) {
+                bx = fma2(c3, dx, bx);
+                by = fma2(c3, dy, by);
+                bz = fma2(c3, dz, bz);
+            }
+            ax[k] = fma2(c3, dx, ax[k]);
+            ay[k] = fma2(c3, dy, ay[k]);
+            az[k] = fma2(c3, dz, az[k]);
+        }
+        if (BOTH) {
+            bx = __shfl_sync(0xffffffffu, bx, src);
+            by = __shfl_sync(0xffffffffu, by, src);
+            bz = __shfl_sync(0xffffffffu, bz, src);
+        }
+    }
+    if (BOTH) {
+        upk2(bx, b[0], b[3]);
+        upk2(by, b[1], b[4]);
+        upk2(bz, b[2], b[5]);
+    }
+}
+
+// Sources per combine step of a CTA of NW warps and tiles of TI ions: the warps meet at two
+// barriers per step, so the step is long (as far as 24 KB of staging allow).
+template <int NW, int TI>
+constexpr int SYM_SUB = NW == 1 ? SYM_GRP : TI < 2048 / NW ? TI : 2048 / NW < 512 ? 2048 / NW : 512;
+
+// what a CTA's symmetric units need of shared memory
+template <int NW, int TI>
+struct SymShared {
+    float acc[3][NW][NW == 1 ? 1 : SYM_SUB<NW, TI>];  // the warps' source-side sums of a step
+    float4 sj[NW * 32];
+    WarpStage stage[NW];
+};
 
 // One tile-pair unit (I, J >= I) of the symmetric kernel with packed FP32 pairs: the same
-// units, fixed-point sums and fixed combine order as k_forces_sym, but the travelling packet holds
-// two sources (the lane's sources q*64 + lane and q*64 + 32 + lane of the group), each
-// target is duplicated into both halves of a pair, and every FP32 operation of the pair
-// term acts on the two sources in one instruction.  Source-side sums are accumulated
-// with the target-side sign and negated when the warps' sums are combined.  Every unit
-// starts on combine buffer 0 and ends on buffer 1, so consecutive units need no barrier
-// between them beyond the one per combine step.
+// units and fixed-point sums as k_forces_sym, the sources in groups of 64 through sym2_group.
+// The warps' source-side sums are added in warp order.  They are accumulated with the
+// target-side sign and negated there.  The caller has a barrier between two units of a CTA.
 template <int BT, int IPT, bool CUT = false>
 __device__ __forceinline__ void sym2_unit(const float4* __restrict__ fpos, const ForceArgs& F, int I, int J,
-                                          float (&s_acc)[2][3][BT / 32][SYM_SUB], float4* sj)
+                                          SymShared<BT / 32, BT * IPT>& S)
 {
     constexpr int NW = BT / 32;
     constexpr int TI = BT * IPT;
-    static_assert(TI % SYM_SUB == 0 && (TI / SYM_SUB) % 2 == 0, "tile must hold an even number of combine steps");
+    constexpr int SUB = SYM_SUB<NW, TI>;
+    static_assert(TI % SUB == 0 && SUB % SYM_GRP == 0, "tile must hold whole combine steps");
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int src = (lane + 1) & 31;
     float xi[IPT], yi[IPT], zi[IPT], ax[IPT], ay[IPT], az[IPT];
 #pragma unroll
     for (int k = 0; k < IPT; ++k) {
@@ -373,68 +453,43 @@ __device__ __forceinline__ void sym2_unit(const float4* __restrict__ fpos, const
         az[k] = 0.f;
     }
     if (I == J) {
-        pair_chunk<BT, IPT, CUT>(fpos, I * TI, I * TI + TI, xi, yi, zi, ax, ay, az, sj, F.cut_s0, F.cut_inv_w);
+        pair_chunk<BT, IPT, CUT>(fpos, I * TI, I * TI + TI, xi, yi, zi, ax, ay, az, S.sj, F.cut_s0, F.cut_inv_w);
     } else {
-        f32x2 xd[IPT], yd[IPT], zd[IPT], ax2[IPT], ay2[IPT], az2[IPT];
+        f32x2 ax2[IPT], ay2[IPT], az2[IPT];
 #pragma unroll
-        for (int k = 0; k < IPT; ++k) {
-            xd[k] = pk2(xi[k], xi[k]);
-            yd[k] = pk2(yi[k], yi[k]);
-            zd[k] = pk2(zi[k], zi[k]);
-            ax2[k] = ay2[k] = az2[k] = 0ull;
-        }
-        const int jb = J * TI;
-        for (int sc = 0; sc < TI / SYM_SUB; ++sc) {
-            const int buf = sc & 1;
+        for (int k = 0; k < IPT; ++k) ax2[k] = ay2[k] = az2[k] = 0ull;
 #pragma unroll 1
-            for (int q = 0; q < SYM_SUB / 64; ++q) {
-                const int j0 = jb + sc * SYM_SUB + q * 64 + lane;
-                const float4 pa = __ldg(fpos + j0), pb = __ldg(fpos + j0 + 32);
-                f32x2 xj = pk2(pa.x, pb.x), yj = pk2(pa.y, pb.y), zj = pk2(pa.z, pb.z);
-                f32x2 bx = 0ull, by = 0ull, bz = 0ull;
-#pragma unroll 2
-                for (int r = 0; r < 32; ++r) {
+        for (int sc = 0; sc < TI / SUB; ++sc) {
+            const int jb = J * TI + sc * SUB;
+            if (NW > 1 && sc > 0) __syncthreads();  // the previous step's sums have been read
+#pragma unroll 1
+            for (int q = 0; q < SUB / SYM_GRP; ++q) {
+                const int jq = q * SYM_GRP + lane;
+                float b[6];
+                sym2_group<IPT, CUT, true>(__ldg(fpos + jb + jq), __ldg(fpos + jb + jq + 32), xi, yi, zi, ax2, ay2,
+                                           az2, b, S.stage[w], F.cut_s0, F.cut_inv_w);
+                if (NW == 1) {
+                    fixed_add3(F.psum, F.psum_ld, jb + jq, -b[0], -b[1], -b[2], F.qscale, F.err);
+                    fixed_add3(F.psum, F.psum_ld, jb + jq + 32, -b[3], -b[4], -b[5], F.qscale, F.err);
+                } else {
 #pragma unroll
-                    for (int k = 0; k < IPT; ++k) {
-                        const f32x2 dx = sub2(xj, xd[k]), dy = sub2(yj, yd[k]), dz = sub2(zj, zd[k]);
-                        const f32x2 c3 = CUT ? pair_c3x2_cut(dx, dy, dz, F.cut_s0, F.cut_inv_w) : pair_c3x2(dx, dy, dz);
-                        ax2[k] = fma2(c3, dx, ax2[k]);
-                        ay2[k] = fma2(c3, dy, ay2[k]);
-                        az2[k] = fma2(c3, dz, az2[k]);
-                        bx = fma2(c3, dx, bx);
-                        by = fma2(c3, dy, by);
-                        bz = fma2(c3, dz, bz);
+                    for (int c = 0; c < 3; ++c) {
+                        S.acc[c][w][jq] = b[c];
+                        S.acc[c][w][jq + 32] = b[3 + c];
                     }
-                    xj = __shfl_sync(0xffffffffu, xj, src);
-                    yj = __shfl_sync(0xffffffffu, yj, src);
-                    zj = __shfl_sync(0xffffffffu, zj, src);
-                    bx = __shfl_sync(0xffffffffu, bx, src);
-                    by = __shfl_sync(0xffffffffu, by, src);
-                    bz = __shfl_sync(0xffffffffu, bz, src);
                 }
-                float l0, h0;
-                upk2(bx, l0, h0);
-                s_acc[buf][0][w][q * 64 + lane] = l0;
-                s_acc[buf][0][w][q * 64 + 32 + lane] = h0;
-                upk2(by, l0, h0);
-                s_acc[buf][1][w][q * 64 + lane] = l0;
-                s_acc[buf][1][w][q * 64 + 32 + lane] = h0;
-                upk2(bz, l0, h0);
-                s_acc[buf][2][w][q * 64 + lane] = l0;
-                s_acc[buf][2][w][q * 64 + 32 + lane] = h0;
             }
-            // one barrier per combine step: the other buffer's readers (previous step)
-            // finished before they reached it
+            if (NW == 1) continue;
             __syncthreads();
-            for (int j = threadIdx.x; j < SYM_SUB; j += BT) {
+            for (int j = threadIdx.x; j < SUB; j += BT) {
                 float sx = 0.f, sy = 0.f, sz = 0.f;
 #pragma unroll
                 for (int ww = 0; ww < NW; ++ww) {
-                    sx += s_acc[buf][0][ww][j];
-                    sy += s_acc[buf][1][ww][j];
-                    sz += s_acc[buf][2][ww][j];
+                    sx += S.acc[0][ww][j];
+                    sy += S.acc[1][ww][j];
+                    sz += S.acc[2][ww][j];
                 }
-                fixed_add3(F.psum, F.psum_ld, jb + sc * SYM_SUB + j, -sx, -sy, -sz, F.qscale, F.err);
+                fixed_add3(F.psum, F.psum_ld, jb + j, -sx, -sy, -sz, F.qscale, F.err);
             }
         }
 #pragma unroll
@@ -455,11 +510,10 @@ __device__ __forceinline__ void sym2_unit(const float4* __restrict__ fpos, const
 
 // Dynamic unit queue: a persistent CTA takes the next unit index from sched[0] (the
 // fixed-point sums are order-independent, so which CTA evaluates a unit changes no
-// result); the last CTA to
-// finish resets both words for the next launch on the stream.
+// result); the last CTA to finish resets both words for the next launch on the stream.
 __device__ __forceinline__ long long next_unit(unsigned long long* sched, long long& s_u)
 {
-    __syncthreads();  // every thread has read the previous index
+    __syncthreads();  // every thread has read the previous index, and the unit's shared sums
     if (threadIdx.x == 0) s_u = (long long)atomicAdd(sched, 1ull);
     __syncthreads();
     return s_u;
@@ -474,26 +528,23 @@ __device__ __forceinline__ void leave_queue(unsigned long long* sched)
 }
 
 // Persistent symmetric kernel on packed FP32 pairs: tile-pair units from the dynamic
-// queue.  The 8-target variants are held to 128 registers (a few spills) for one more
-// resident CTA per SM, which measured 1% faster than their natural 133.
+// queue.  The 8-target variants run 12 warps per SM with up to 168 registers.
 template <int BT, int IPT>
-__global__ void __launch_bounds__(BT, (IPT == 8 ? 65536 / (BT * 128) : 1))
+__global__ void __launch_bounds__(BT, (IPT == 8 ? 65536 / (BT * 168) : 1))
     k_forces_sym2(const float4* __restrict__ fpos, ForceArgs F)
 {
     constexpr int TI = BT * IPT;
-    __shared__ float s_acc[2][3][BT / 32][SYM_SUB];
-    __shared__ float4 sj[BT];
+    __shared__ SymShared<BT / 32, TI> S;
     __shared__ long long s_u;
     // tiles from the live count on hold only far-away dummies, whose terms with live ions
-    // are exactly zero: units that reach such a tile (J >= I) are skipped.  The count is read again for every unit (a volatile load),
-    // so that it takes no register across the unit's code, which sits at the register cap.
+    // are exactly zero: units that reach such a tile (J >= I) are skipped
     for (;;) {
         const long long u = next_unit(F.sched, s_u);
         if (u >= F.U) break;
         int I, J;
         tri_unit(u, F.JS, I, J);
         if (F.n_live && J * TI >= *(volatile const int*)F.n_live) continue;
-        sym2_unit<BT, IPT>(fpos, F, I, J, s_acc, sj);
+        sym2_unit<BT, IPT>(fpos, F, I, J, S);
     }
     leave_queue(F.sched);
 }
