@@ -10,18 +10,20 @@
 //   h4_k = relu(W4 h3_k + b4)           256
 //   y_k  = W5 h4_k + b5                 4 outputs (padded to 16)
 // Weights are kept in FP32 (master copy for Adam) and used as BF16 in every matrix
-// product (BF16 inputs, FP32 accumulation: tcgen05.mma tiles by default, od_gemm_tc.cu,
-// or warp-level mma.sync m16n8k16 tiles, k_gemm_nt below);
-// activations are rounded to BF16 where they enter a product.  The loss is the mean
-// squared error over present grains and the four outputs.
+// product (BF16 inputs, FP32 accumulation); activations are rounded to BF16 where they enter
+// a product.  The loss is the mean squared error over present grains and the four outputs.
+// By default the network runs as the fused kernels of od_mlp.cu on the fifth-generation tensor
+// cores.  OD_GEMM_MMA_SYNC runs it layer by layer with warp-level mma.sync products
+// (k_gemm_nt and the kernels below) as an independent cross-check.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
 #include <vector>
 
-#include "od_internal.h"
+#include "od_mlp.cuh"
 
 namespace od {
 namespace sur {
@@ -183,13 +185,41 @@ __global__ void k_unpool(const float* __restrict__ dx3, const float* __restrict_
     da2[i] = dx3[(long long)row * 2 * H + j] + share;
 }
 
-// Adam on FP32 master parameters, then the BF16 copy (and its transpose for weights)
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                       __nv_bfloat16* __restrict__ pb, __nv_bfloat16* __restrict__ pbt, int rows, int cols, float lr,
-                       float b1, float b2, float eps, float c1, float c2)
+// where parameter i of the flat vector lives in the BF16 copies: the element of wb (out x in per
+// layer, one after another) and of wt (its transpose); false for a bias
+__device__ __forceinline__ bool weight_place(int i, int& wb, int& wt)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)rows * cols) return;
+    int base = 0;  // weights of the layers before
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {
+        const int rows = mlp::out_of(l), cols = mlp::in_of(l), k = i - mlp::w_off(l);
+        if (k < rows * (cols + 1)) {
+            wb = base + k;
+            wt = base + (k % cols) * rows + k / cols;
+            return k < rows * cols;
+        }
+        base += rows * cols;
+    }
+    return false;
+}
+
+// the BF16 copies of the weights and their transposes from the FP32 masters
+__global__ void k_refresh(const float* __restrict__ p, __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int a, b;
+    if (i >= mlp::N_PARAMS || !weight_place(i, a, b)) return;
+    wb[a] = wt[b] = __float2bfloat16_rn(p[i]);
+}
+
+// Adam on the FP32 master parameters, then the BF16 copies of the weights: one launch over the
+// whole vector
+__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
+                       __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt, float lr, float b1, float b2,
+                       float eps, float c1, float c2)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= mlp::N_PARAMS) return;
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
@@ -197,11 +227,39 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
     v[i] = vi;
     const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     p[i] = pi;
-    if (pb) pb[i] = __float2bfloat16_rn(pi);
-    if (pbt) {
-        const int r = (int)(i / cols), c = (int)(i % cols);
-        pbt[(long long)c * rows + r] = __float2bfloat16_rn(pi);
+    int a, b;
+    if (weight_place(i, a, b)) wb[a] = wt[b] = __float2bfloat16_rn(pi);
+}
+
+// the loss: row losses added in FP64 in a fixed order (one CTA)
+__global__ void __launch_bounds__(256) k_loss_sum(const float* __restrict__ row_loss, int rows, double* __restrict__ loss)
+{
+    __shared__ double s[256];
+    double a = 0.0;
+    for (int r = threadIdx.x; r < rows; r += 256) a += (double)row_loss[r];
+    s[threadIdx.x] = a;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
+        __syncthreads();
     }
+    if (threadIdx.x == 0) *loss = s[0];
+}
+
+// inputs padded to K0 columns for the layer-by-layer products
+__global__ void k_pad_inputs(const float* __restrict__ x, __nv_bfloat16* __restrict__ x0, int M)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M * K0) return;
+    const int r = i / K0, c = i % K0;
+    x0[i] = __float2bfloat16_rn(c < IN ? x[r * IN + c] : 0.f);
+}
+
+// the four real outputs of the padded output layer
+__global__ void k_take_outputs(const float* __restrict__ y, float* __restrict__ out, int M)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < M * OUTR) out[i] = y[(i / OUTR) * OUTP + i % OUTR];
 }
 
 }  // namespace sur
@@ -215,24 +273,41 @@ namespace {
 
 struct Layer {
     int out, in;
-    float *w = nullptr, *b = nullptr;        // FP32 master
-    float *gw = nullptr, *gb = nullptr;      // gradients
-    float *mw = nullptr, *vw = nullptr, *mb = nullptr, *vb = nullptr;  // Adam moments
+    float *w = nullptr, *b = nullptr;            // FP32 master, in the flat parameter vector
+    float *gw = nullptr, *gb = nullptr;          // gradients, likewise
     __nv_bfloat16 *wb = nullptr, *wt = nullptr;  // BF16 copy [out][in] and transpose [in][out]
 };
 
 }  // namespace
 
+// results the host reads after a pass
+struct SurOut {
+    double loss;
+    int err;  // tensor-core wait timeouts (bit 1)
+    int pad;
+};
+
 struct od_sur {
-    int maxB = 0;
+    int maxB = 0, sms = 0;
     Layer L[5];
-    // activations, M = maxB * G rows
-    __nv_bfloat16 *x0b, *h1b, *h2b, *x3b, *h3b, *h4b, *dyb, *dzb, *tA, *tB;
-    float *h1, *h2, *c, *h3, *h4, *y, *dy, *dx, *dx3, *da, *rowl, *mask, *tgt, *xin;
+    float *p = nullptr, *g = nullptr, *am = nullptr, *av = nullptr;  // parameters, gradients, Adam moments
+    __nv_bfloat16 *wb = nullptr, *wt = nullptr;
+    // inputs, outputs and the fused pass's activations, rows padded to whole tiles
+    float *x = nullptr, *mask = nullptr, *tgt = nullptr, *y = nullptr, *rowl = nullptr, *dbias = nullptr, *part = nullptr;
+    mlp::Acts acts{};
+    mlp::FusedMaps fmaps;
+    mlp::GradMaps gmaps;
+    SurOut* d_out = nullptr;
+    SurOut* h_out = nullptr;  // page-locked
+    // layer-by-layer engine, allocated when it is first selected (M = maxB * G rows)
+    bool layers = false;
+    __nv_bfloat16 *x0b = nullptr, *h1b = nullptr, *h2b = nullptr, *x3b = nullptr, *h3b = nullptr, *h4b = nullptr,
+                  *dyb = nullptr, *dzb = nullptr, *tA = nullptr, *tB = nullptr;
+    float *h1 = nullptr, *h2 = nullptr, *c = nullptr, *h3 = nullptr, *h4 = nullptr, *yp = nullptr, *dy = nullptr,
+          *dx3 = nullptr, *da = nullptr;
     cudaStream_t stream = nullptr;
     long long adam_t = 0;
     int engine = OD_GEMM_TCGEN05;
-    int* d_err = nullptr;  // tensor-core wait timeouts (bit 1)
     std::string err;
 };
 
@@ -273,21 +348,21 @@ int gemm_bf16(const __nv_bfloat16* A, const __nv_bfloat16* B, const float* bias,
 
 namespace {
 
+// a product of the layer-by-layer engine
 int gemm(od_sur* s, const __nv_bfloat16* A, const __nv_bfloat16* B, const float* bias, float* C, __nv_bfloat16* Cb, int M,
          int N, int K, int relu)
 {
-    const int e = gemm_bf16(A, B, bias, C, Cb, M, N, K, relu, s->engine, s->d_err, s->stream);
+    const int e = gemm_bf16(A, B, bias, C, Cb, M, N, K, relu, OD_GEMM_MMA_SYNC, &s->d_out->err, s->stream);
     return e == 0 ? OD_OK : sfail(s, OD_ECUDA, std::string("gemm launch failed: ") + cudaGetErrorString((cudaError_t)e));
 }
 
-// tensor-core waits that gave up since the last check (read after a synchronisation)
-int check_engine(od_sur* s)
+// the pass's loss and error word, after everything queued on the stream
+int read_out(od_sur* s)
 {
-    int e = 0;
-    SCK(s, cudaMemcpyAsync(&e, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    SCK(s, cudaMemcpyAsync(s->h_out, s->d_out, sizeof(SurOut), cudaMemcpyDeviceToHost, s->stream));
     SCK(s, cudaStreamSynchronize(s->stream));
-    if (e) {
-        SCK(s, cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream));
+    if (s->h_out->err) {
+        SCK(s, cudaMemsetAsync(s->d_out, 0, sizeof(SurOut), s->stream));
         return sfail(s, OD_ETIMEOUT, "a tensor-core product's wait gave up");
     }
     return OD_OK;
@@ -295,43 +370,58 @@ int check_engine(od_sur* s)
 
 void free_sur(od_sur* s)
 {
-    for (auto& l : s->L) {
-        cudaFree(l.w), cudaFree(l.b), cudaFree(l.gw), cudaFree(l.gb), cudaFree(l.mw), cudaFree(l.vw), cudaFree(l.mb),
-            cudaFree(l.vb), cudaFree(l.wb), cudaFree(l.wt);
-    }
-    void* bufs[] = {s->x0b, s->h1b, s->h2b, s->x3b, s->h3b, s->h4b, s->dyb, s->dzb, s->tA, s->tB, s->h1, s->h2,
-                    s->c, s->h3, s->h4, s->y, s->dy, s->dx, s->dx3, s->da, s->rowl, s->mask, s->tgt, s->xin};
+    void* bufs[] = {s->p, s->g, s->am, s->av, s->wb, s->wt, s->x, s->mask, s->tgt, s->y, s->rowl, s->dbias, s->part,
+                    s->acts.x0, s->acts.h1, s->acts.x3, s->acts.h3, s->acts.h4, s->acts.dy, s->acts.dz4, s->acts.dz3,
+                    s->acts.dz2, s->acts.dz1, s->d_out, s->x0b, s->h1b, s->h2b, s->x3b, s->h3b, s->h4b, s->dyb, s->dzb,
+                    s->tA, s->tB, s->h1, s->h2, s->c, s->h3, s->h4, s->yp, s->dy, s->dx3, s->da};
     for (void* p : bufs) cudaFree(p);
-    cudaFree(s->d_err);
+    cudaFreeHost(s->h_out);
+}
+
+// buffers of the layer-by-layer engine
+int ensure_layers(od_sur* s)
+{
+    if (s->layers) return OD_OK;
+    const long long M = (long long)s->maxB * G;
+    struct {
+        void** p;
+        long long bytes;
+    } want[] = {{(void**)&s->x0b, 2 * M * K0}, {(void**)&s->h1b, 2 * M * H}, {(void**)&s->h2b, 2 * M * H},
+                {(void**)&s->x3b, 4 * M * H},  {(void**)&s->h3b, 2 * M * H}, {(void**)&s->h4b, 2 * M * H},
+                {(void**)&s->dyb, 2 * M * OUTP}, {(void**)&s->dzb, 2 * M * H}, {(void**)&s->tA, 4 * M * H},
+                {(void**)&s->tB, 4 * M * H},   {(void**)&s->h1, 4 * M * H},  {(void**)&s->h2, 4 * M * H},
+                {(void**)&s->c, 4 * s->maxB * (long long)H}, {(void**)&s->h3, 4 * M * H}, {(void**)&s->h4, 4 * M * H},
+                {(void**)&s->yp, 4 * M * OUTP}, {(void**)&s->dy, 4 * M * OUTP}, {(void**)&s->dx3, 8 * M * H},
+                {(void**)&s->da, 8 * M * H}};
+    for (auto& w : want)
+        if (!*w.p && cudaMalloc(w.p, w.bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return sfail(s, OD_ENOMEM, "surrogate: no memory for the layer-by-layer engine");
+        }
+    s->layers = true;
+    return OD_OK;
 }
 
 // refresh the BF16 copies of every layer from the FP32 masters
 int refresh_bf16(od_sur* s)
 {
-    for (auto& l : s->L) {
-        const long long n = (long long)l.out * l.in;
-        k_to_bf16<<<blocks(n), 256, 0, s->stream>>>(l.w, l.wb, n);
-        k_transpose<<<blocks(n), 256, 0, s->stream>>>(l.wb, l.wt, l.out, l.in);
-    }
+    k_refresh<<<blocks(mlp::N_PARAMS), 256, 0, s->stream>>>(s->p, s->wb, s->wt);
     return cudaGetLastError() == cudaSuccess ? OD_OK : sfail(s, OD_ECUDA, "weight refresh failed");
 }
 
-// inputs: xin [B][G][IN] FP32 (host layout copied), mask [B][G]
-int forward(od_sur* s, int Bn)
+// forward pass layer by layer (rows a multiple of 16)
+int forward_layers(od_sur* s, int Bn)
 {
     const int M = Bn * G;
-    // x0 padded to K0 columns
-    {
-        std::vector<float> dummy;  // padding is done on the host when uploading
-    }
     int rc;
+    k_pad_inputs<<<blocks((long long)M * K0), 256, 0, s->stream>>>(s->x, s->x0b, M);
     if ((rc = gemm(s, s->x0b, s->L[0].wb, s->L[0].b, s->h1, s->h1b, M, H, K0, 1))) return rc;
     if ((rc = gemm(s, s->h1b, s->L[1].wb, s->L[1].b, s->h2, s->h2b, M, H, H, 1))) return rc;
     k_pool<<<blocks((long long)Bn * H), 256, 0, s->stream>>>(s->h2, s->mask, s->c, Bn);
     k_concat<<<blocks((long long)M * 2 * H), 256, 0, s->stream>>>(s->h2b, s->c, s->x3b, M);
     if ((rc = gemm(s, s->x3b, s->L[2].wb, s->L[2].b, s->h3, s->h3b, M, H, 2 * H, 1))) return rc;
     if ((rc = gemm(s, s->h3b, s->L[3].wb, s->L[3].b, s->h4, s->h4b, M, H, H, 1))) return rc;
-    if ((rc = gemm(s, s->h4b, s->L[4].wb, s->L[4].b, s->y, nullptr, M, OUTP, H, 0))) return rc;
+    if ((rc = gemm(s, s->h4b, s->L[4].wb, s->L[4].b, s->yp, nullptr, M, OUTP, H, 0))) return rc;
     return OD_OK;
 }
 
@@ -346,10 +436,11 @@ int weight_grad(od_sur* s, Layer& l, const float* dz, const __nv_bfloat16* dzb, 
     return OD_OK;
 }
 
-int backward(od_sur* s, int Bn)
+int backward_layers(od_sur* s, int Bn, float inv_count)
 {
     const int M = Bn * G;
     int rc;
+    k_loss<<<blocks(M), 256, 0, s->stream>>>(s->yp, s->tgt, s->mask, s->dy, s->rowl, M, inv_count);
     // output layer: dy (FP32) -> BF16
     k_to_bf16<<<blocks((long long)M * OUTP), 256, 0, s->stream>>>(s->dy, s->dyb, (long long)M * OUTP);
     if ((rc = weight_grad(s, s->L[4], s->dy, s->dyb, s->h4b, M))) return rc;
@@ -370,38 +461,78 @@ int backward(od_sur* s, int Bn)
     return cudaGetLastError() == cudaSuccess ? OD_OK : sfail(s, OD_ECUDA, "backward launch failed");
 }
 
+// the batch's arrays as they come; the layer-by-layer engine takes an even number of samples,
+// the last of an odd batch absent and zero
 int upload_batch(od_sur* s, const float* x, const float* mask, const float* tgt, int Bn)
 {
-    const int M = Bn * G;
-    std::vector<float> xp((size_t)M * K0, 0.f);
-    for (int r = 0; r < M; ++r)
-        for (int j = 0; j < IN; ++j) xp[(size_t)r * K0 + j] = x[(size_t)r * IN + j];
-    SCK(s, cudaMemcpyAsync(s->xin, xp.data(), sizeof(float) * xp.size(), cudaMemcpyHostToDevice, s->stream));
-    k_to_bf16<<<blocks((long long)M * K0), 256, 0, s->stream>>>(s->xin, s->x0b, (long long)M * K0);
+    const size_t M = (size_t)Bn * G;
+    SCK(s, cudaMemcpyAsync(s->x, x, sizeof(float) * M * IN, cudaMemcpyHostToDevice, s->stream));
     SCK(s, cudaMemcpyAsync(s->mask, mask, sizeof(float) * M, cudaMemcpyHostToDevice, s->stream));
     if (tgt) SCK(s, cudaMemcpyAsync(s->tgt, tgt, sizeof(float) * M * OUTR, cudaMemcpyHostToDevice, s->stream));
+    if (s->engine == OD_GEMM_MMA_SYNC && Bn % 2) {
+        SCK(s, cudaMemsetAsync(s->x + M * IN, 0, sizeof(float) * G * IN, s->stream));
+        SCK(s, cudaMemsetAsync(s->mask + M, 0, sizeof(float) * G, s->stream));
+        SCK(s, cudaMemsetAsync(s->tgt + M * OUTR, 0, sizeof(float) * G * OUTR, s->stream));
+    }
     return OD_OK;
 }
 
-int loss_and_grad(od_sur* s, int Bn, const float* mask_host, double* loss)
+mlp::FusedArgs fused_args(od_sur* s, int Bn)
 {
-    const int M = Bn * G;
-    double cnt = 0.0;
-    for (int r = 0; r < M; ++r) cnt += mask_host[r] > 0.f ? 1.0 : 0.0;
-    const float inv = cnt > 0 ? (float)(1.0 / (cnt * OUTR)) : 0.f;
-    int rc = forward(s, Bn);
-    if (rc) return rc;
-    k_loss<<<blocks(M), 256, 0, s->stream>>>(s->y, s->tgt, s->mask, s->dy, s->rowl, M, inv);
-    if ((rc = backward(s, Bn))) return rc;
-    if (loss) {
-        std::vector<float> rl(M);
-        SCK(s, cudaMemcpyAsync(rl.data(), s->rowl, sizeof(float) * M, cudaMemcpyDeviceToHost, s->stream));
-        SCK(s, cudaStreamSynchronize(s->stream));
-        double l = 0.0;
-        for (float v : rl) l += v;
-        *loss = l;
+    mlp::FusedArgs A{};
+    A.x = s->x;
+    A.mask = s->mask;
+    A.tgt = s->tgt;
+    for (int l = 0; l < 5; ++l) A.bias[l] = s->L[l].b;
+    A.y = s->y;
+    A.row_loss = s->rowl;
+    A.dbias = s->dbias;
+    A.x0 = s->acts.x0;
+    A.dy = s->acts.dy;
+    A.rows = Bn * G;
+    A.tiles = (A.rows + mlp::TILE - 1) / mlp::TILE;
+    A.err = &s->d_out->err;
+    return A;
+}
+
+// outputs of the uploaded batch into s->y [rows][4]
+int run_forward(od_sur* s, int Bn)
+{
+    if (s->engine == OD_GEMM_MMA_SYNC) {
+        const int Bp = (Bn + 1) / 2 * 2;
+        const int rc = forward_layers(s, Bp);
+        if (rc) return rc;
+        k_take_outputs<<<blocks((long long)Bp * G * OUTR), 256, 0, s->stream>>>(s->yp, s->y, Bp * G);
+        return cudaGetLastError() == cudaSuccess ? OD_OK : sfail(s, OD_ECUDA, "forward launch failed");
     }
-    return OD_OK;
+    const int e = mlp::launch_forward(s->fmaps, fused_args(s, Bn), s->sms, s->stream);
+    return e == 0 ? OD_OK : sfail(s, OD_ECUDA, std::string("forward launch failed: ") + cudaGetErrorString((cudaError_t)e));
+}
+
+// loss and gradients of the uploaded batch into d_out and the gradient vector
+int run_gradients(od_sur* s, int Bn, const float* mask_host)
+{
+    long long cnt = 0;
+    for (int r = 0; r < Bn * G; ++r) cnt += mask_host[r] > 0.f;
+    const float inv = cnt > 0 ? (float)(1.0 / ((double)cnt * OUTR)) : 0.f;
+    int rows = Bn * G, rc, e;
+    if (s->engine == OD_GEMM_MMA_SYNC) {
+        const int Bp = (Bn + 1) / 2 * 2;
+        rows = Bp * G;
+        if ((rc = forward_layers(s, Bp)) || (rc = backward_layers(s, Bp, inv))) return rc;
+    } else {
+        mlp::FusedArgs A = fused_args(s, Bn);
+        A.y = nullptr;
+        A.inv_count = inv;
+        const int splits = mlp::grad_splits(rows, s->sms);
+        int ctas = 0;
+        if ((e = mlp::launch_forward_backward(s->fmaps, A, s->sms, &ctas, s->stream)) ||
+            (e = mlp::launch_weight_grads(s->gmaps, s->part, rows, splits, &s->d_out->err, s->stream)) ||
+            (e = mlp::launch_grad_reduce(s->part, splits, s->dbias, ctas * mlp::QUADS, s->g, s->stream)))
+            return sfail(s, OD_ECUDA, std::string("gradient launch failed: ") + cudaGetErrorString((cudaError_t)e));
+    }
+    k_loss_sum<<<1, 256, 0, s->stream>>>(s->rowl, rows, &s->d_out->loss);
+    return cudaGetLastError() == cudaSuccess ? OD_OK : sfail(s, OD_ECUDA, "loss launch failed");
 }
 
 }  // namespace
@@ -415,10 +546,11 @@ int od_sur_create(int max_batch, uint64_t seed, void* stream, od_sur** out)
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) return sfail(nullptr, OD_ENODEV, "no CUDA device");
     od_sur* s = new od_sur();
-    std::memset((void*)&s->x0b, 0, sizeof(void*) * 24);
-    s->maxB = (max_batch + 1) / 2 * 2;  // M = 8 B rows must be a multiple of 16
+    s->maxB = (max_batch + 1) / 2 * 2;  // the layer-by-layer engine takes whole pairs of samples
     s->stream = (cudaStream_t)stream;
-    const int dims[5][2] = {{H, K0}, {H, H}, {H, 2 * H}, {H, H}, {OUTP, H}};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev);
     // He-uniform initial weights from a seeded host generator (splitmix64), zero biases
     unsigned long long st = seed * 0x9E3779B97F4A7C15ull + 12345ull;
     auto next = [&st]() {
@@ -428,67 +560,78 @@ int od_sur_create(int max_batch, uint64_t seed, void* stream, od_sur** out)
         return z ^ (z >> 31);
     };
     bool ok = true;
-    for (int li = 0; li < 5 && ok; ++li) {
-        Layer& l = s->L[li];
-        l.out = dims[li][0];
-        l.in = dims[li][1];
-        const size_t nw = (size_t)l.out * l.in;
-        const int fan_in = li == 0 ? IN : l.in;
-        const double bound = std::sqrt(6.0 / fan_in) * (li == 4 ? 0.1 : 1.0);
-        std::vector<float> w(nw, 0.f);
-        for (int o = 0; o < l.out; ++o)
-            for (int i = 0; i < l.in; ++i) {
-                const bool live = (li != 0 || i < IN) && (li != 4 || o < OUTR);
-                const double u = (double)(next() >> 11) * (1.0 / 9007199254740992.0);
-                w[(size_t)o * l.in + i] = live ? (float)((2.0 * u - 1.0) * bound) : 0.f;
-            }
-        ok = cudaMalloc(&l.w, sizeof(float) * nw) == cudaSuccess && cudaMalloc(&l.b, sizeof(float) * l.out) == cudaSuccess &&
-             cudaMalloc(&l.gw, sizeof(float) * nw) == cudaSuccess && cudaMalloc(&l.gb, sizeof(float) * l.out) == cudaSuccess &&
-             cudaMalloc(&l.mw, sizeof(float) * nw) == cudaSuccess && cudaMalloc(&l.vw, sizeof(float) * nw) == cudaSuccess &&
-             cudaMalloc(&l.mb, sizeof(float) * l.out) == cudaSuccess && cudaMalloc(&l.vb, sizeof(float) * l.out) == cudaSuccess &&
-             cudaMalloc(&l.wb, sizeof(__nv_bfloat16) * nw) == cudaSuccess &&
-             cudaMalloc(&l.wt, sizeof(__nv_bfloat16) * nw) == cudaSuccess;
-        if (!ok) break;
-        cudaMemcpyAsync(l.w, w.data(), sizeof(float) * nw, cudaMemcpyHostToDevice, s->stream);
-        cudaMemsetAsync(l.b, 0, sizeof(float) * l.out, s->stream);
-        cudaMemsetAsync(l.mw, 0, sizeof(float) * nw, s->stream);
-        cudaMemsetAsync(l.vw, 0, sizeof(float) * nw, s->stream);
-        cudaMemsetAsync(l.mb, 0, sizeof(float) * l.out, s->stream);
-        cudaMemsetAsync(l.vb, 0, sizeof(float) * l.out, s->stream);
-    }
-    const long long M = (long long)s->maxB * G;
     auto mb = [&](void** p, size_t bytes) { ok = ok && cudaMalloc(p, bytes) == cudaSuccess; };
-    mb((void**)&s->x0b, 2 * M * K0);
-    mb((void**)&s->h1b, 2 * M * H);
-    mb((void**)&s->h2b, 2 * M * H);
-    mb((void**)&s->x3b, 2 * M * 2 * H);
-    mb((void**)&s->h3b, 2 * M * H);
-    mb((void**)&s->h4b, 2 * M * H);
-    mb((void**)&s->dyb, 2 * M * OUTP);
-    mb((void**)&s->dzb, 2 * M * H);
-    mb((void**)&s->tA, 2 * M * 2 * H);
-    mb((void**)&s->tB, 2 * M * 2 * H);
-    mb((void**)&s->h1, 4 * M * H);
-    mb((void**)&s->h2, 4 * M * H);
-    mb((void**)&s->c, 4 * (long long)s->maxB * H);
-    mb((void**)&s->h3, 4 * M * H);
-    mb((void**)&s->h4, 4 * M * H);
-    mb((void**)&s->y, 4 * M * OUTP);
-    mb((void**)&s->dy, 4 * M * OUTP);
-    mb((void**)&s->dx, 4 * M * H);
-    mb((void**)&s->dx3, 4 * M * 2 * H);
-    mb((void**)&s->da, 4 * M * 2 * H);
-    mb((void**)&s->rowl, 4 * M);
+    mb((void**)&s->p, sizeof(float) * mlp::N_PARAMS);
+    mb((void**)&s->g, sizeof(float) * mlp::N_PARAMS);
+    mb((void**)&s->am, sizeof(float) * mlp::N_PARAMS);
+    mb((void**)&s->av, sizeof(float) * mlp::N_PARAMS);
+    mb((void**)&s->wb, sizeof(__nv_bfloat16) * mlp::N_PARAMS);
+    mb((void**)&s->wt, sizeof(__nv_bfloat16) * mlp::N_PARAMS);
+    const long long M = ((long long)s->maxB * G + mlp::TILE - 1) / mlp::TILE * mlp::TILE;  // rows in whole tiles
+    mb((void**)&s->x, 4 * M * IN);
     mb((void**)&s->mask, 4 * M);
     mb((void**)&s->tgt, 4 * M * OUTR);
-    mb((void**)&s->xin, 4 * M * K0);
-    mb((void**)&s->d_err, sizeof(int));
-    if (ok) ok = cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream) == cudaSuccess;
-    if (!ok || refresh_bf16(s) != OD_OK || cudaStreamSynchronize(s->stream) != cudaSuccess) {
+    mb((void**)&s->y, 4 * M * OUTR);
+    mb((void**)&s->rowl, 4 * M);
+    mb((void**)&s->dbias, sizeof(float) * mlp::QUADS * mlp::BIAS_LD * (size_t)s->sms);
+    mb((void**)&s->part, sizeof(float) * mlp::N_PARAMS * (size_t)mlp::grad_splits((int)std::min(M, 16384ll), s->sms));
+    mb((void**)&s->acts.x0, 2 * M * K0);
+    mb((void**)&s->acts.h1, 2 * M * H);
+    mb((void**)&s->acts.x3, 4 * M * H);
+    mb((void**)&s->acts.h3, 2 * M * H);
+    mb((void**)&s->acts.h4, 2 * M * H);
+    mb((void**)&s->acts.dy, 2 * M * OUTP);
+    mb((void**)&s->acts.dz4, 2 * M * H);
+    mb((void**)&s->acts.dz3, 2 * M * H);
+    mb((void**)&s->acts.dz2, 2 * M * H);
+    mb((void**)&s->acts.dz1, 2 * M * H);
+    mb((void**)&s->d_out, sizeof(SurOut));
+    ok = ok && cudaMallocHost((void**)&s->h_out, sizeof(SurOut)) == cudaSuccess;
+    if (ok) {
+        std::vector<float> p(mlp::N_PARAMS, 0.f);
+        long long wo = 0;
+        for (int li = 0; li < 5; ++li) {
+            Layer& l = s->L[li];
+            l.out = mlp::out_of(li);
+            l.in = mlp::in_of(li);
+            const int off = mlp::w_off(li), nw = l.out * l.in;
+            l.w = s->p + off;
+            l.b = l.w + nw;
+            l.gw = s->g + off;
+            l.gb = l.gw + nw;
+            l.wb = s->wb + wo;
+            l.wt = s->wt + wo;
+            wo += nw;
+            const int fan_in = li == 0 ? IN : l.in;
+            const double bound = std::sqrt(6.0 / fan_in) * (li == 4 ? 0.1 : 1.0);
+            for (int o = 0; o < l.out; ++o)
+                for (int i = 0; i < l.in; ++i) {
+                    const bool live = (li != 0 || i < IN) && (li != 4 || o < OUTR);
+                    const double u = (double)(next() >> 11) * (1.0 / 9007199254740992.0);
+                    p[(size_t)off + o * l.in + i] = live ? (float)((2.0 * u - 1.0) * bound) : 0.f;
+                }
+        }
+        cudaMemcpyAsync(s->p, p.data(), sizeof(float) * p.size(), cudaMemcpyHostToDevice, s->stream);
+        cudaMemsetAsync(s->g, 0, sizeof(float) * p.size(), s->stream);
+        cudaMemsetAsync(s->am, 0, sizeof(float) * p.size(), s->stream);
+        cudaMemsetAsync(s->av, 0, sizeof(float) * p.size(), s->stream);
+        ok = cudaMemsetAsync(s->d_out, 0, sizeof(SurOut), s->stream) == cudaSuccess &&
+             refresh_bf16(s) == OD_OK && cudaStreamSynchronize(s->stream) == cudaSuccess;
+    }
+    if (!ok) {
+        cudaGetLastError();
         g_sur_error = "surrogate allocation failed";
         free_sur(s);
         delete s;
         return OD_ENOMEM;
+    }
+    const __nv_bfloat16 *wb[5], *wt[5];
+    for (int l = 0; l < 5; ++l) wb[l] = s->L[l].wb, wt[l] = s->L[l].wt;
+    if (!mlp::encode_maps(wb, wt, s->acts, (int)M, s->fmaps, s->gmaps)) {
+        g_sur_error = "surrogate: tensor map encoding failed";
+        free_sur(s);
+        delete s;
+        return OD_ECUDA;
     }
     *out = s;
     return OD_OK;
@@ -503,25 +646,13 @@ void od_sur_destroy(od_sur* s)
     delete s;
 }
 
-int od_sur_num_params(const od_sur* s)
-{
-    if (!s) return 0;
-    int n = 0;
-    for (const auto& l : s->L) n += l.out * l.in + l.out;
-    return n;
-}
+int od_sur_num_params(const od_sur* s) { return s ? mlp::N_PARAMS : 0; }
 
 // FP32 master parameters, layer by layer: W (out x in, row-major) then b (out)
 int od_sur_get_params(od_sur* s, float* host)
 {
     if (!s || !host) return sfail(s, OD_EINVAL, "bad argument");
-    size_t off = 0;
-    for (auto& l : s->L) {
-        SCK(s, cudaMemcpyAsync(host + off, l.w, sizeof(float) * l.out * l.in, cudaMemcpyDeviceToHost, s->stream));
-        off += (size_t)l.out * l.in;
-        SCK(s, cudaMemcpyAsync(host + off, l.b, sizeof(float) * l.out, cudaMemcpyDeviceToHost, s->stream));
-        off += l.out;
-    }
+    SCK(s, cudaMemcpyAsync(host, s->p, sizeof(float) * mlp::N_PARAMS, cudaMemcpyDeviceToHost, s->stream));
     SCK(s, cudaStreamSynchronize(s->stream));
     return OD_OK;
 }
@@ -529,13 +660,7 @@ int od_sur_get_params(od_sur* s, float* host)
 int od_sur_set_params(od_sur* s, const float* host)
 {
     if (!s || !host) return sfail(s, OD_EINVAL, "bad argument");
-    size_t off = 0;
-    for (auto& l : s->L) {
-        SCK(s, cudaMemcpyAsync(l.w, host + off, sizeof(float) * l.out * l.in, cudaMemcpyHostToDevice, s->stream));
-        off += (size_t)l.out * l.in;
-        SCK(s, cudaMemcpyAsync(l.b, host + off, sizeof(float) * l.out, cudaMemcpyHostToDevice, s->stream));
-        off += l.out;
-    }
+    SCK(s, cudaMemcpyAsync(s->p, host, sizeof(float) * mlp::N_PARAMS, cudaMemcpyHostToDevice, s->stream));
     int rc = refresh_bf16(s);
     if (rc) return rc;
     SCK(s, cudaStreamSynchronize(s->stream));
@@ -546,44 +671,25 @@ int od_sur_set_params(od_sur* s, const float* host)
 int od_sur_forward(od_sur* s, const float* x, const float* mask, int Bn, float* y)
 {
     if (!s || !x || !mask || !y || Bn < 1 || Bn > s->maxB) return sfail(s, OD_EINVAL, "bad forward arguments");
-    const int Bp = (Bn + 1) / 2 * 2, M = Bp * G;
-    std::vector<float> xs((size_t)M * IN, 0.f), ms(M, 0.f);
-    std::memcpy(xs.data(), x, sizeof(float) * Bn * G * IN);
-    std::memcpy(ms.data(), mask, sizeof(float) * Bn * G);
-    int rc = upload_batch(s, xs.data(), ms.data(), nullptr, Bp);
+    int rc = upload_batch(s, x, mask, nullptr, Bn);
     if (rc) return rc;
-    if ((rc = forward(s, Bp))) return rc;
-    std::vector<float> yy((size_t)M * OUTP);
-    SCK(s, cudaMemcpyAsync(yy.data(), s->y, sizeof(float) * yy.size(), cudaMemcpyDeviceToHost, s->stream));
-    if ((rc = check_engine(s))) return rc;
-    for (int r = 0; r < Bn * G; ++r)
-        for (int o = 0; o < OUTR; ++o) y[(size_t)r * OUTR + o] = yy[(size_t)r * OUTP + o];
-    return OD_OK;
+    if ((rc = run_forward(s, Bn))) return rc;
+    SCK(s, cudaMemcpyAsync(y, s->y, sizeof(float) * Bn * G * OUTR, cudaMemcpyDeviceToHost, s->stream));
+    return read_out(s);
 }
 
 // loss and parameter gradients (layout of od_sur_get_params) without an update
 int od_sur_gradients(od_sur* s, const float* x, const float* mask, const float* tgt, int Bn, double* loss, float* grads)
 {
     if (!s || !x || !mask || !tgt || Bn < 1 || Bn > s->maxB) return sfail(s, OD_EINVAL, "bad gradient arguments");
-    const int Bp = (Bn + 1) / 2 * 2, M = Bp * G;
-    std::vector<float> xs((size_t)M * IN, 0.f), ms(M, 0.f), ts((size_t)M * OUTR, 0.f);
-    std::memcpy(xs.data(), x, sizeof(float) * Bn * G * IN);
-    std::memcpy(ms.data(), mask, sizeof(float) * Bn * G);
-    std::memcpy(ts.data(), tgt, sizeof(float) * Bn * G * OUTR);
-    int rc = upload_batch(s, xs.data(), ms.data(), ts.data(), Bp);
+    int rc = upload_batch(s, x, mask, tgt, Bn);
     if (rc) return rc;
-    if ((rc = loss_and_grad(s, Bp, ms.data(), loss))) return rc;
-    if (loss && (rc = check_engine(s))) return rc;
-    if (grads) {
-        size_t off = 0;
-        for (auto& l : s->L) {
-            SCK(s, cudaMemcpyAsync(grads + off, l.gw, sizeof(float) * l.out * l.in, cudaMemcpyDeviceToHost, s->stream));
-            off += (size_t)l.out * l.in;
-            SCK(s, cudaMemcpyAsync(grads + off, l.gb, sizeof(float) * l.out, cudaMemcpyDeviceToHost, s->stream));
-            off += l.out;
-        }
-        if ((rc = check_engine(s))) return rc;
-    }
+    if ((rc = run_gradients(s, Bn, mask))) return rc;
+    if (grads)
+        SCK(s, cudaMemcpyAsync(grads, s->g, sizeof(float) * mlp::N_PARAMS, cudaMemcpyDeviceToHost, s->stream));
+    if (!grads && !loss) return OD_OK;
+    if ((rc = read_out(s))) return rc;
+    if (loss) *loss = s->h_out->loss;
     return OD_OK;
 }
 
@@ -595,12 +701,7 @@ int od_sur_train_step(od_sur* s, const float* x, const float* mask, const float*
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     s->adam_t += 1;
     const float c1 = 1.f - std::pow(b1, (float)s->adam_t), c2 = 1.f - std::pow(b2, (float)s->adam_t);
-    for (auto& l : s->L) {
-        const long long nw = (long long)l.out * l.in;
-        k_adam<<<blocks(nw), 256, 0, s->stream>>>(l.w, l.gw, l.mw, l.vw, l.wb, l.wt, l.out, l.in, lr, b1, b2, eps, c1, c2);
-        k_adam<<<blocks(l.out), 256, 0, s->stream>>>(l.b, l.gb, l.mb, l.vb, nullptr, nullptr, 1, l.out, lr, b1, b2, eps, c1,
-                                                      c2);
-    }
+    k_adam<<<blocks(mlp::N_PARAMS), 256, 0, s->stream>>>(s->p, s->g, s->am, s->av, s->wb, s->wt, lr, b1, b2, eps, c1, c2);
     if (cudaGetLastError() != cudaSuccess) return sfail(s, OD_ECUDA, "adam launch failed");
     return OD_OK;
 }
@@ -610,6 +711,10 @@ const char* od_sur_last_error(const od_sur* s) { return s ? s->err.c_str() : g_s
 int od_sur_set_gemm(od_sur* s, int engine)
 {
     if (!s || (engine != OD_GEMM_TCGEN05 && engine != OD_GEMM_MMA_SYNC)) return sfail(s, OD_EINVAL, "bad engine");
+    if (engine == OD_GEMM_MMA_SYNC) {
+        const int rc = ensure_layers(s);
+        if (rc) return rc;
+    }
     s->engine = engine;
     return OD_OK;
 }

@@ -1,0 +1,39 @@
+"""The fused network kernels (128-row tiles of 16 samples; weight gradients over ranges of 64-row
+chunks) at the edges of their tiles and ranges, against the layer-by-layer mma.sync engine.
+
+Both engines round the same values to BF16 and accumulate in FP32 in different orders, so a sum
+that lies on a rounding boundary may round differently; the bars are those the two engines meet
+against the FP64 reference (outputs 1e-3 of the largest, gradients 5e-3 of each block's norm).
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B", [1, 15, 16, 17, 129, 2049])  # less than a tile .. two ranges of rows
+def test_fused_kernels_agree_with_the_layer_by_layer_engine(B):
+    import paper_2205_06557_gb300 as od
+
+    rng = np.random.default_rng(B)
+    x = rng.uniform(-1.0, 1.0, (B, 8, 7))
+    mask = (rng.uniform(size=(B, 8)) < 0.5).astype(np.float64)
+    mask[:, 0] = 1.0
+    if B > 2:
+        mask[2] = 0.0  # a sample without grains
+    t = rng.normal(size=(B, 8, 4))
+    s = od.Surrogate(max_batch=B, seed=B)
+    out = {}
+    for eng in (od.GEMM_MMA_SYNC, od.GEMM_TCGEN05):
+        s.set_gemm(eng)
+        out[eng] = (s.forward(x, mask), *s.gradients(x, mask, t))
+    s.close()
+    (y0, l0, g0), (y1, l1, g1) = out[od.GEMM_MMA_SYNC], out[od.GEMM_TCGEN05]
+    assert np.abs(y1 - y0).max() <= 1e-3 * np.abs(y0).max()
+    assert abs(l1 - l0) <= 1e-4 * abs(l0)
+    off = 0
+    for o, i in od.Surrogate.SHAPES:
+        for n in (o * i, o):
+            a, b = g1[off: off + n].astype(np.float64), g0[off: off + n].astype(np.float64)
+            off += n
+            assert np.linalg.norm(a - b) <= 5e-3 * np.linalg.norm(b), (o, i, n)
