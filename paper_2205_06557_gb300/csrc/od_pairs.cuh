@@ -59,6 +59,99 @@ __device__ __forceinline__ float pair_c3_cut(float dx, float dy, float dz, float
     return (e * (ri * ri)) * switch_bracket(s, ri, s0, w_inv);
 }
 
+// ---------------------------------------- packed FP32 pairs (f32x2, sm_100 family)
+// Two FP32 values in one 64-bit register pair; add/sub/mul/fma on both in one
+// instruction with the same IEEE round-to-nearest as the scalar forms.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pk2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+__device__ __forceinline__ void upk2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// pair_c3 for two pairs at once (same operations and rounding per lane of the pair)
+__device__ __forceinline__ f32x2 pair_c3x2(f32x2 dx, f32x2 dy, f32x2 dz)
+{
+    const f32x2 eps2 = pk2(1e-24f, 1e-24f), ln2 = pk2(0.69314718055994531f, 0.69314718055994531f);
+    f32x2 r2 = fma2(dx, dx, eps2);
+    r2 = fma2(dy, dy, r2);
+    r2 = fma2(dz, dz, r2);
+    float ra, rb;
+    upk2(r2, ra, rb);
+    const f32x2 ri = pk2(rsqrt_approx(ra), rsqrt_approx(rb));
+    float sa, sb;
+    upk2(mul2(r2, ri), sa, sb);
+    const f32x2 e = pk2(ex2_approx(-sa), ex2_approx(-sb));
+    return mul2(mul2(e, mul2(ri, ri)), add2(ri, ln2));
+}
+
+// switch_bracket for two pairs at once, in packed operations (only the clamp is per
+// lane): x = (s - s0) w_inv in [0, 1], S = 1 + x^3 (15 x - 6 x^2 - 10),
+// -S' = 30 x^2 (1 - x)^2, bracket = (ri + ln2) S + 30 w_inv x^2 (1 - x)^2
+__device__ __forceinline__ f32x2 switch_bracket2(f32x2 s, f32x2 ri, float s0, float w_inv)
+{
+    constexpr float LN2 = 0.69314718055994531f;
+    f32x2 x = fma2(s, pk2(w_inv, w_inv), pk2(-s0 * w_inv, -s0 * w_inv));
+    float xa, xb;
+    upk2(x, xa, xb);
+    x = pk2(fminf(fmaxf(xa, 0.f), 1.f), fminf(fmaxf(xb, 0.f), 1.f));
+    const f32x2 x2 = mul2(x, x);
+    const f32x2 t = fma2(fma2(x, pk2(-6.f, -6.f), pk2(15.f, 15.f)), x, pk2(-10.f, -10.f));
+    const f32x2 S = fma2(mul2(x2, x), t, pk2(1.f, 1.f));
+    const f32x2 y2 = fma2(x, add2(x, pk2(-2.f, -2.f)), pk2(1.f, 1.f));
+    return fma2(mul2(x2, y2), pk2(30.f * w_inv, 30.f * w_inv), mul2(add2(ri, pk2(LN2, LN2)), S));
+}
+
+// pair_c3_cut for two pairs at once: the packed plain coefficient's steps, then the
+// packed switching bracket
+__device__ __forceinline__ f32x2 pair_c3x2_cut(f32x2 dx, f32x2 dy, f32x2 dz, float s0, float w_inv)
+{
+    const f32x2 eps2 = pk2(1e-24f, 1e-24f);
+    f32x2 r2 = fma2(dx, dx, eps2);
+    r2 = fma2(dy, dy, r2);
+    r2 = fma2(dz, dz, r2);
+    float ra, rb;
+    upk2(r2, ra, rb);
+    const f32x2 ri = pk2(rsqrt_approx(ra), rsqrt_approx(rb));
+    const f32x2 s = mul2(r2, ri);
+    float sa, sb;
+    upk2(s, sa, sb);
+    const f32x2 e = pk2(ex2_approx(-sa), ex2_approx(-sb));
+    return mul2(mul2(e, mul2(ri, ri)), switch_bracket2(s, ri, s0, w_inv));
+}
+
 // Accumulate into IPT targets per thread the pair terms of sources [j0, j1), staged
 // through shared memory BT at a time (acc += d c3, c3 from pair_c3, or from pair_c3_cut
 // with the switching zone s0, w_inv when CUT).
@@ -132,6 +225,41 @@ __global__ void __launch_bounds__(BT) k_forces(const float4* __restrict__ fpos, 
         float4* out = part + (long long)slot * F.n_pad + t * F.TI + threadIdx.x;
 #pragma unroll
         for (int k = 0; k < IPT; ++k) out[k * BT] = make_float4(ax[k], ay[k], az[k], 0.f);
+    }
+}
+
+// ------------------------------------------------- ordered pairs on packed FP32 pairs
+// One warp: 256 targets, eight per lane, against NS pairs of sources read by every lane
+// from shared memory; an f32x2 holds the terms of the two sources of a pair.  The sums (from
+// zero) of the first and of the second sources stay apart in the halves.  Per ordered pair 14
+// FP32 operations beside a MUFU rsqrt and ex2.  (Two targets per f32x2 and one source were
+// slower: half the independent chains per lane.)
+constexpr int ORD_T = 8;  // targets per lane
+
+template <int NS>
+struct SourcePairs {
+    f32x2 x[NS], y[NS], z[NS];
+};
+
+template <int NS>
+__device__ __forceinline__ void ordered_pairs(const SourcePairs<NS>& S, const float (&xi)[ORD_T],
+                                              const float (&yi)[ORD_T], const float (&zi)[ORD_T], f32x2 (&bx)[ORD_T],
+                                              f32x2 (&by)[ORD_T], f32x2 (&bz)[ORD_T])
+{
+#pragma unroll
+    for (int k = 0; k < ORD_T; ++k) bx[k] = by[k] = bz[k] = 0ull;
+#pragma unroll 4
+    for (int jj = 0; jj < NS; ++jj) {
+        const f32x2 xj = S.x[jj], yj = S.y[jj], zj = S.z[jj];
+#pragma unroll
+        for (int k = 0; k < ORD_T; ++k) {
+            const f32x2 dx = sub2(xj, pk2(xi[k], xi[k])), dy = sub2(yj, pk2(yi[k], yi[k])),
+                        dz = sub2(zj, pk2(zi[k], zi[k]));
+            const f32x2 c3 = pair_c3x2(dx, dy, dz);
+            bx[k] = fma2(c3, dx, bx[k]);
+            by[k] = fma2(c3, dy, by[k]);
+            bz[k] = fma2(c3, dz, bz[k]);
+        }
     }
 }
 
@@ -247,99 +375,6 @@ __global__ void __launch_bounds__(BT) k_forces_sym(const float4* __restrict__ fp
             fixed_add3(F.psum, F.psum_ld, I * TI + k * BT + threadIdx.x, ax[k], ay[k], az[k], F.qscale, F.err);
         if (++J == T) J = ++I;
     }
-}
-
-// ---------------------------------------- packed FP32 pairs (f32x2, sm_100 family)
-// Two FP32 values in one 64-bit register pair; add/sub/mul/fma on both in one
-// instruction with the same IEEE round-to-nearest as the scalar forms.
-typedef unsigned long long f32x2;
-
-__device__ __forceinline__ f32x2 pk2(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-
-__device__ __forceinline__ void upk2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
-{
-    f32x2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-// pair_c3 for two pairs at once (same operations and rounding per lane of the pair)
-__device__ __forceinline__ f32x2 pair_c3x2(f32x2 dx, f32x2 dy, f32x2 dz)
-{
-    const f32x2 eps2 = pk2(1e-24f, 1e-24f), ln2 = pk2(0.69314718055994531f, 0.69314718055994531f);
-    f32x2 r2 = fma2(dx, dx, eps2);
-    r2 = fma2(dy, dy, r2);
-    r2 = fma2(dz, dz, r2);
-    float ra, rb;
-    upk2(r2, ra, rb);
-    const f32x2 ri = pk2(rsqrt_approx(ra), rsqrt_approx(rb));
-    float sa, sb;
-    upk2(mul2(r2, ri), sa, sb);
-    const f32x2 e = pk2(ex2_approx(-sa), ex2_approx(-sb));
-    return mul2(mul2(e, mul2(ri, ri)), add2(ri, ln2));
-}
-
-// switch_bracket for two pairs at once, in packed operations (only the clamp is per
-// lane): x = (s - s0) w_inv in [0, 1], S = 1 + x^3 (15 x - 6 x^2 - 10),
-// -S' = 30 x^2 (1 - x)^2, bracket = (ri + ln2) S + 30 w_inv x^2 (1 - x)^2
-__device__ __forceinline__ f32x2 switch_bracket2(f32x2 s, f32x2 ri, float s0, float w_inv)
-{
-    constexpr float LN2 = 0.69314718055994531f;
-    f32x2 x = fma2(s, pk2(w_inv, w_inv), pk2(-s0 * w_inv, -s0 * w_inv));
-    float xa, xb;
-    upk2(x, xa, xb);
-    x = pk2(fminf(fmaxf(xa, 0.f), 1.f), fminf(fmaxf(xb, 0.f), 1.f));
-    const f32x2 x2 = mul2(x, x);
-    const f32x2 t = fma2(fma2(x, pk2(-6.f, -6.f), pk2(15.f, 15.f)), x, pk2(-10.f, -10.f));
-    const f32x2 S = fma2(mul2(x2, x), t, pk2(1.f, 1.f));
-    const f32x2 y2 = fma2(x, add2(x, pk2(-2.f, -2.f)), pk2(1.f, 1.f));
-    return fma2(mul2(x2, y2), pk2(30.f * w_inv, 30.f * w_inv), mul2(add2(ri, pk2(LN2, LN2)), S));
-}
-
-// pair_c3_cut for two pairs at once: the packed plain coefficient's steps, then the
-// packed switching bracket
-__device__ __forceinline__ f32x2 pair_c3x2_cut(f32x2 dx, f32x2 dy, f32x2 dz, float s0, float w_inv)
-{
-    const f32x2 eps2 = pk2(1e-24f, 1e-24f);
-    f32x2 r2 = fma2(dx, dx, eps2);
-    r2 = fma2(dy, dy, r2);
-    r2 = fma2(dz, dz, r2);
-    float ra, rb;
-    upk2(r2, ra, rb);
-    const f32x2 ri = pk2(rsqrt_approx(ra), rsqrt_approx(rb));
-    const f32x2 s = mul2(r2, ri);
-    float sa, sb;
-    upk2(s, sa, sb);
-    const f32x2 e = pk2(ex2_approx(-sa), ex2_approx(-sb));
-    return mul2(mul2(e, mul2(ri, ri)), switch_bracket2(s, ri, s0, w_inv));
 }
 
 // ------------------------------------------- symmetric units on packed FP32 pairs
