@@ -631,33 +631,29 @@ int launch_density(od_handle* h)
     return OD_OK;
 }
 
-// the next step's injection samples on the second stream, beside the pair forces (fork
-// after the scan, which fixes their ids; joined by join_ahead before the step ends)
-// and this step's collision velocities on a third (joined by join_collide before the kick)
-int fork_ahead(od_handle* h)
+// what runs beside the pair forces, on three more streams (forked after the scan): the ion
+// terms the kick adds (joined by join_terms before it), the grain side and the next step's
+// injection samples (joined by join_rest before the step ends)
+int fork_beside(od_handle* h)
 {
-    if (!h->aux) return OD_OK;
     OD_CK(h, cudaEventRecord(h->ev_fork, h->stream));
-    OD_CK(h, cudaStreamWaitEvent(h->aux, h->ev_fork, 0));
-    OD_LK(h, launch_inject_ahead(h->P, h->B, h->aux));
-    OD_CK(h, cudaEventRecord(h->ev_join, h->aux));
-    OD_CK(h, cudaStreamWaitEvent(h->aux2, h->ev_fork, 0));
-    OD_LK(h, launch_collide_ahead(h->P, h->B, h->aux2));
-    OD_CK(h, cudaEventRecord(h->ev_join2, h->aux2));
+    for (int k = 0; k < 3; ++k) OD_CK(h, cudaStreamWaitEvent(h->aux[k], h->ev_fork, 0));
+    OD_LK(h, launch_ion_terms(h->P, h->B, h->aux[0]));
+    OD_LK(h, launch_grains(h->P, h->B, h->aux[1]));
+    OD_LK(h, launch_inject_ahead(h->P, h->B, h->aux[2]));
+    for (int k = 0; k < 3; ++k) OD_CK(h, cudaEventRecord(h->ev_join[k], h->aux[k]));
     return OD_OK;
 }
 
-int join_collide(od_handle* h)
+int join_terms(od_handle* h)
 {
-    if (!h->aux) return OD_OK;
-    OD_CK(h, cudaStreamWaitEvent(h->stream, h->ev_join2, 0));
+    OD_CK(h, cudaStreamWaitEvent(h->stream, h->ev_join[0], 0));
     return OD_OK;
 }
 
-int join_ahead(od_handle* h)
+int join_rest(od_handle* h)
 {
-    if (!h->aux) return OD_OK;
-    OD_CK(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
+    for (int k = 1; k < 3; ++k) OD_CK(h, cudaStreamWaitEvent(h->stream, h->ev_join[k], 0));
     return OD_OK;
 }
 
@@ -665,11 +661,11 @@ int launch_step(od_handle* h)
 {
     int rc;
     OD_LK(h, launch_push_scan(h->P, h->B, h->stream));
-    if ((rc = fork_ahead(h))) return rc;
+    if ((rc = fork_beside(h))) return rc;
     OD_LK(h, launch_pairs(h, 1));
-    if ((rc = join_collide(h))) return rc;
-    OD_LK(h, launch_kick(h->P, h->B, h->F, 0, h->stream));  // with the grain tail
-    if ((rc = join_ahead(h))) return rc;
+    if ((rc = join_terms(h))) return rc;
+    OD_LK(h, launch_kick_step(h->P, h->B, h->F, h->stream));
+    if ((rc = join_rest(h))) return rc;
     return launch_density(h);
 }
 
@@ -776,11 +772,13 @@ void free_all(od_handle* h)
         if (e) cudaEventDestroy(e);
     cudaFree(h->B.inj_ahead);
     cudaFree(h->B.coll_v);
+    cudaFree(h->B.pre);
+    cudaFree(h->B.felt);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
-    if (h->ev_join) cudaEventDestroy(h->ev_join);
-    if (h->ev_join2) cudaEventDestroy(h->ev_join2);
-    if (h->aux) cudaStreamDestroy(h->aux);
-    if (h->aux2) cudaStreamDestroy(h->aux2);
+    for (auto& e : h->ev_join)
+        if (e) cudaEventDestroy(e);
+    for (auto& s : h->aux)
+        if (s) cudaStreamDestroy(s);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 
@@ -804,8 +802,9 @@ int create_impl(const od_params* p, od_handle* h)
     {
         std::vector<double> tab;
         build_vtab(h->P.u, h->P.sig, tab, h->P.gmax_b, h->P.gmax_t);
-        OD_CK(h, cudaMalloc(&h->d_vtab, sizeof(double) * tab.size()));
+        OD_CK(h, cudaMalloc(&h->d_vtab, sizeof(double) * (tab.size() + 2)));
         OD_CK(h, cudaMemcpyAsync(h->d_vtab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice, h->stream));
+        OD_LK(h, launch_vtab_consts(h->d_vtab, h->P.u, h->P.sig, h->stream));
         OD_CK(h, cudaStreamSynchronize(h->stream));
         h->P.vtab = h->d_vtab;
     }
@@ -861,14 +860,16 @@ int create_impl(const od_params* p, od_handle* h)
     OD_CK(h, cudaMalloc(&B.rem, sizeof(Rem) * h->cap));
     OD_CK(h, cudaMalloc(&B.inj_ahead, sizeof(Inj) * INJ_AHEAD));
     if (!h->batch_member) {
-        // single runs draw the next step's injection samples and this step's collision
-        // velocities on two more streams, beside the pair forces
+        // single runs compute what does not need the pair forces beside them, on more streams
         OD_CK(h, cudaMalloc(&B.coll_v, sizeof(double) * 3 * h->cap));
-        OD_CK(h, cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking));
-        OD_CK(h, cudaStreamCreateWithFlags(&h->aux2, cudaStreamNonBlocking));
+        OD_CK(h, cudaMalloc(&B.pre, sizeof(double) * 6 * h->cap));
+        OD_CK(h, cudaMalloc(&B.felt, sizeof(Felt)));
+        OD_CK(h, cudaMemsetAsync(B.felt, 0, sizeof(Felt), h->stream));
         OD_CK(h, cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
-        OD_CK(h, cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
-        OD_CK(h, cudaEventCreateWithFlags(&h->ev_join2, cudaEventDisableTiming));
+        for (int k = 0; k < 3; ++k) {
+            OD_CK(h, cudaStreamCreateWithFlags(&h->aux[k], cudaStreamNonBlocking));
+            OD_CK(h, cudaEventCreateWithFlags(&h->ev_join[k], cudaEventDisableTiming));
+        }
     }
     OD_CK(h, cudaMalloc(&B.dpart, sizeof(double) * h->nb_cap * MAXD * 3));
     OD_CK(h, cudaMalloc(&B.ctrl, sizeof(Ctrl)));
@@ -1007,14 +1008,14 @@ int od_step(od_handle* h, int64_t n)
                 OD_CK(h, cudaEventRecord(e[0], h->stream));
                 OD_LK(h, launch_push_scan(h->P, h->B, h->stream));
                 OD_CK(h, cudaEventRecord(e[1], h->stream));
-                if ((rc = fork_ahead(h))) return rc;
+                if ((rc = fork_beside(h))) return rc;
                 OD_LK(h, launch_pairs(h, 1));
                 OD_CK(h, cudaEventRecord(e[2], h->stream));
-                if ((rc = join_collide(h))) return rc;
-                OD_LK(h, launch_kick(h->P, h->B, h->F, 0, h->stream));  // with the grain tail
+                if ((rc = join_terms(h))) return rc;
+                OD_LK(h, launch_kick_step(h->P, h->B, h->F, h->stream));
                 OD_CK(h, cudaEventRecord(e[3], h->stream));
                 OD_CK(h, cudaEventRecord(e[4], h->stream));
-                if ((rc = join_ahead(h))) return rc;
+                if ((rc = join_rest(h))) return rc;
                 if ((rc = launch_density(h))) return rc;
                 if (++h->pev_used == PROF_RING && (rc = drain_profile(h))) return rc;
             } else {

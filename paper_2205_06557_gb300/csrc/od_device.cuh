@@ -58,18 +58,17 @@ __device__ __forceinline__ double npdf(double z) { return exp(-0.5 * z * z) * 0.
 // derivative |v| N(v; u, s^2), kept inside a shrinking bracket (bisection when a step
 // leaves it).  The bottom face's flux up to axial speed v is
 //   int_0^v v' N(v'; u, s^2) dv' = u (Phi(z) - Phi(z0)) + s (phi(z0) - phi(z)),
-// the top face's from v < 0 up to 0 is -u (Phi(z0) - Phi(z)) + s (phi(z0) - phi(z)), with
-// z = (v - u) / s, z0 = -u / s (Phi, phi the standard normal CDF and density); Phi(z0)
-// and phi(z0) are evaluated once per sample, Phi(z) and phi(z) once per iteration.
-template <bool TOP>
-__device__ double invert_flux(double target, double lo, double hi, double v, double u, double s)
+// the top face's from v < 0 up to 0 is the same expression, decreasing in v, with
+// z = (v - u) / s, z0 = -u / s (Phi, phi the standard normal CDF and density; c0 = Phi(z0)
+// and p0 = phi(z0) are the run's constants).
+static __device__ double invert_flux(bool top, double target, double lo, double hi, double v, double u, double s,
+                                     double c0, double p0)
 {
-    const double z0 = -u / s, c0 = ncdf(z0), p0 = npdf(z0);
     for (int it = 0; it < 100; ++it) {
         const double z = (v - u) / s;
         const double cz = ncdf(z), pz = npdf(z);
-        const double F = TOP ? -u * (c0 - cz) + s * (p0 - pz) : u * (cz - c0) + s * (p0 - pz);
-        const double g = TOP ? (target - F) : (F - target);  // increasing in v
+        const double F = u * (cz - c0) + s * (p0 - pz);
+        const double g = top ? (target - F) : (F - target);  // increasing in v
         if (g < 0) lo = v;
         else hi = v;
         const double dg = fabs(v) * pz / s;
@@ -91,52 +90,78 @@ __device__ double invert_flux(double target, double lo, double hi, double v, dou
     return v;
 }
 
-// App. B: face by flux probability, position uniform on the face, flux-weighted velocity
+// App. B: face by flux probability, position uniform on the face, flux-weighted velocity.
+// The sample's independent FP64 draws, from the Philox words A (ST_INJ_A) and the normals'
+// words Bw (ST_INJ_B); inj_assemble puts them together.  FP64 is slow on this GPU and each
+// draw is a long dependent chain, so the sampler that runs ahead gives each to a warp of its
+// own (k_inject_ahead).
+__device__ __forceinline__ int inj_face(const Phys& P, uint4 A)
+{
+    return (unsigned long long)A.x < P.Tb ? 0 : (unsigned long long)A.x < P.Tbt ? 1 : 2;
+}
+
+__device__ __forceinline__ void inj_angle(int face, uint4 A, double& s, double& c)
+{
+    sincos(6.283185307179586 * unif(face == 2 ? A.y : A.z), &s, &c);
+}
+
+// axial speed through a cap: the tabulated inverse CDF brackets the root and gives the
+// starting point, Newton polishes it to ~1e-13 (a few iterations instead of a bisection
+// from the whole range)
+__device__ __forceinline__ double inj_axial(const Phys& P, int face, uint4 A)
+{
+    const double U = unif(A.w);
+    const double xk = U * VTAB_K;
+    const int k = min((int)xk, VTAB_K - 1);
+    const double* tab = P.vtab + (face == 0 ? 0 : VTAB_K + 1);
+    const double t0 = tab[k], t1 = tab[k + 1];
+    const double c0 = P.vtab[2 * (VTAB_K + 1)], p0 = P.vtab[2 * (VTAB_K + 1) + 1];
+    const double pad = 1e-12 * fmax(fmax(fabs(t0), fabs(t1)), P.sig);
+    const double v0 = t0 + (xk - k) * (t1 - t0);
+    double lo = fmin(t0, t1) - pad, hi = fmax(t0, t1) + pad;
+    if (face == 0) lo = fmax(lo, 0.0);
+    else hi = fmin(hi, 0.0);
+    return invert_flux(face == 1, U * (face == 0 ? P.gmax_b : P.gmax_t), lo, hi, v0, P.u, P.sig, c0, p0);
+}
+
+// flux-weighted radial speed through the side (Rayleigh)
+__device__ __forceinline__ double inj_radial(const Phys& P, uint4 A) { return P.sig * sqrt(-2.0 * log(unif(A.w))); }
+
+// n0, n1: normals; s, c: the angle's sine and cosine; sp: the axial (caps) or radial speed
+__device__ __forceinline__ void inj_assemble(const Phys& P, unsigned long long id, int face, uint4 A, double n0,
+                                             double n1, double s, double c, double sp, Inj& o)
+{
+    if (face != 2) {
+        const double rho = P.R * sqrt(unif(A.y));
+        o.x = rho * c;
+        o.y = rho * s;
+        o.z = face == 0 ? -0.5 * P.H : 0.5 * P.H;
+        o.vx = P.sig * n0;
+        o.vy = P.sig * n1;
+        o.vz = sp;
+    } else {
+        o.x = P.R * c;
+        o.y = P.R * s;
+        o.z = P.H * (unif(A.z) - 0.5);
+        const double vt = (P.flags & OD_F_PAPER_SIDE) ? 0.0 : P.sig * n0;
+        o.vx = -sp * c - vt * s;
+        o.vy = -sp * s + vt * c;
+        o.vz = P.u + P.sig * n1;
+    }
+    o.face = face;
+    o.id = id;
+}
+
 static __device__ void sample_injection(const Phys& P, unsigned long long id, uint32_t sn, Inj& o)
 {
     const uint4 A = philox(P, id, sn, ST_INJ_A);
     const uint4 Bw = philox(P, id, sn, ST_INJ_B);
-    double n0, n1;
+    const int face = inj_face(P, A);
+    double n0, n1, s, c;
     box_muller(Bw.x, Bw.y, n0, n1);
-    if ((unsigned long long)A.x < P.Tbt) {
-        const int f = (unsigned long long)A.x < P.Tb ? 0 : 1;
-        const double rho = P.R * sqrt(unif(A.y));
-        double s, c;
-        sincos(6.283185307179586 * unif(A.z), &s, &c);
-        o.x = rho * c;
-        o.y = rho * s;
-        o.z = f == 0 ? -0.5 * P.H : 0.5 * P.H;
-        o.vx = P.sig * n0;
-        o.vy = P.sig * n1;
-        // flux-weighted axial speed: the tabulated inverse CDF brackets the root and gives
-        // the starting point, Newton polishes it to ~1e-13 (FP64 is slow on this GPU: a
-        // few iterations instead of a bisection from the whole range)
-        const double U = unif(A.w);
-        const double xk = U * VTAB_K;
-        const int k = min((int)xk, VTAB_K - 1);
-        const double* tab = P.vtab + (f == 0 ? 0 : VTAB_K + 1);
-        const double t0 = tab[k], t1 = tab[k + 1];
-        const double pad = 1e-12 * fmax(fmax(fabs(t0), fabs(t1)), P.sig);
-        const double v0 = t0 + (xk - k) * (t1 - t0);
-        if (f == 0)
-            o.vz = invert_flux<false>(U * P.gmax_b, fmax(fmin(t0, t1) - pad, 0.0), fmax(t0, t1) + pad, v0, P.u, P.sig);
-        else
-            o.vz = invert_flux<true>(U * P.gmax_t, fmin(t0, t1) - pad, fmin(fmax(t0, t1) + pad, 0.0), v0, P.u, P.sig);
-        o.face = f;
-    } else {
-        double s, c;
-        sincos(6.283185307179586 * unif(A.y), &s, &c);
-        o.x = P.R * c;
-        o.y = P.R * s;
-        o.z = P.H * (unif(A.z) - 0.5);
-        const double vr = P.sig * sqrt(-2.0 * log(unif(A.w)));  // Rayleigh: flux-weighted radial speed
-        const double vt = (P.flags & OD_F_PAPER_SIDE) ? 0.0 : P.sig * n0;
-        o.vx = -vr * c - vt * s;
-        o.vy = -vr * s + vt * c;
-        o.vz = P.u + P.sig * n1;
-        o.face = 2;
-    }
-    o.id = id;
+    inj_angle(face, A, s, c);
+    const double sp = face == 2 ? inj_radial(P, A) : inj_axial(P, face, A);
+    inj_assemble(P, id, face, A, n0, n1, s, c, sp, o);
 }
 
 // The App. B sample of the ion with this id entering in step sn: computed ahead (during
@@ -665,6 +690,12 @@ __device__ __forceinline__ void push_scan_body(const Phys& P, const Bufs& B, int
         const float far = 3.0e4f + 7.0f * (float)(d - n_new);
         B.fpos[d] = make_float4(far, far, far, 0.0f);
     }
+    // the step's number and the charges its ions feel, for the kick: the grain tail may change
+    // the control block's before the kick reads them
+    if (B.felt) {
+        if (threadIdx.x == 32) B.felt->step = step;
+        if ((int)threadIdx.x < P.D) B.felt->Q[threadIdx.x] = C->Q[threadIdx.x];
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         C->ev_step[9] += s_face[0];
@@ -698,25 +729,108 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// mode 0: after the push (second half kick + collisions); mode 1: forces only (creation
-// or a replaced ion state)
-template <int BT, int CP_WIDE = 8>
-__device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const ForceArgs& F, int mode, int blk)
+// What a step's kick adds that does not depend on the pair forces, for ion i at (x, y, z):
+// the close-pair correction (scaled units) and the acceleration of E_out (FP64 polynomial)
+// and the driving field.
+template <int CP_WIDE>
+__device__ __forceinline__ void ion_terms(const Phys& P, const Bufs& B, int buf, int i, double x, double y, double z,
+                                          double& cx, double& cy, double& cz, double& bx, double& by, double& bz)
+{
+    const Ctrl* C = B.ctrl;
+    cx = cy = cz = 0.0;
+    if (P.cp_on) {
+        const double* Xb = B.x[buf];
+        const long long cap = B.cap;
+        close_pair_corr<CP_WIDE>(B.cp_head, B.cp_next, B.fpos, P.cp_mask, P.cp_hinv, P.cp_dc2, C->cp_epoch, C->n_cur,
+                                 P.ls_inv, i, x, y, z,
+                                 [&](int j, double& xj, double& yj, double& zj) {
+                                     xj = Xb[j];
+                                     yj = Xb[cap + j];
+                                     zj = Xb[2 * cap + j];
+                                 },
+                                 cx, cy, cz);
+    }
+    bx = by = 0.0;
+    bz = P.qm * P.E;
+    if (P.eout) {
+        double ex, ey, ez;
+        eout_field(P, x, y, z, ex, ey, ez);
+        bx += P.qm * ex;
+        by += P.qm * ey;
+        bz += P.qm * ez;
+    }
+}
+
+// grain side of Eq. 1 without the prefactor q Q_k / (4 pi eps0), over one block of ions:
+// sum_i (1 + rho/lambda) exp(-rho/lambda) (r_k - r_i) / rho^3; FP32 terms from FP64
+// separations, FP64 sums in a fixed order (warp tree, then block tree)
+template <int BT>
+__device__ __forceinline__ void grain_sums(const Phys& P, const Bufs& B, bool live, double x, double y, double z, int blk)
 {
     __shared__ double s_red[BT / 32][3];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float lam_inv = (float)P.lam_inv;
+    const float lam_inv_l2 = (float)(P.lam_inv * 1.4426950408889634);
+    for (int k = 0; k < P.D; ++k) {
+        double fx = 0.0, fy = 0.0, fz = 0.0;
+        if (live) {
+            const float dx = (float)(P.gx[k] - x), dy = (float)(P.gy[k] - y), dz = (float)(P.gz[k] - z);
+            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            const float ri = rsqrt_approx(r2);
+            const float rho = r2 * ri;
+            const float f = fmaf(rho, lam_inv, 1.0f) * ex2_approx(-rho * lam_inv_l2) * (ri * ri * ri);
+            fx = (double)(f * dx);
+            fy = (double)(f * dy);
+            fz = (double)(f * dz);
+        }
+        fx = warp_sum(fx);
+        fy = warp_sum(fy);
+        fz = warp_sum(fz);
+        if (lane == 0) {
+            s_red[warp][0] = fx;
+            s_red[warp][1] = fy;
+            s_red[warp][2] = fz;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            double a0 = lane < BT / 32 ? s_red[lane][0] : 0.0;
+            double a1 = lane < BT / 32 ? s_red[lane][1] : 0.0;
+            double a2 = lane < BT / 32 ? s_red[lane][2] : 0.0;
+            a0 = warp_sum(a0);
+            a1 = warp_sum(a1);
+            a2 = warp_sum(a2);
+            if (lane == 0) {
+                double* o = B.dpart + ((long long)blk * MAXD + k) * 3;
+                o[0] = a0;
+                o[1] = a1;
+                o[2] = a2;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// mode 0: after the push (second half kick + collisions); mode 1: forces only (creation
+// or a replaced ion state).  PRE (single runs' steps): the ion terms, the collision velocities
+// and the grain side have been computed beside the pair forces (Bufs::pre, coll_v; the step
+// number and the charges the ions feel are Bufs::felt's).
+template <int BT, int CP_WIDE = 8, bool PRE = false>
+__device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const ForceArgs& F, int mode, int blk)
+{
     __shared__ double s_Q[MAXD];
     Ctrl* C = B.ctrl;
-    const long long step = C->step;
+    const long long step = PRE ? B.felt->step : C->step;
     const int buf = mode == 0 ? (int)((step + 1) & 1) : (int)(step & 1);
     const uint32_t sn = (uint32_t)(step + 1);
     const int i = blk * BT + threadIdx.x;
     const bool live = i < C->n_cur;
     const long long cap = B.cap;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const bool sym_sums = F.sym && !(P.flags & OD_F_NO_IONION);
     // every load that does not depend on another is issued first (one memory round trip):
-    // position, velocity, id, the fixed-point pair sums, the grain charges
+    // position, velocity, id, the fixed-point pair sums, the ion terms, the grain charges
     double x = 0, y = 0, z = 0, vx = 0, vy = 0, vz = 0;
+    double cx = 0, cy = 0, cz = 0, bx = 0, by = 0, bz = 0;
     unsigned long long id = 0;
     long long qa = 0, qb = 0, qc = 0;
     long long* A = nullptr;
@@ -732,6 +846,11 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
             vz = V[2 * cap + i];
             id = B.id[buf][i];
         }
+        if (PRE) {
+            const double* T = B.pre;
+            cx = __ldcg(T + i), cy = __ldcg(T + cap + i), cz = __ldcg(T + 2 * cap + i);
+            bx = __ldcg(T + 3 * cap + i), by = __ldcg(T + 4 * cap + i), bz = __ldcg(T + 5 * cap + i);
+        }
         if (sym_sums) {
             // symmetric kernels (all pairs or the cutoff's listed tile pairs): the fixed-point
             // sum at the ion's position in the pair kernel's order (cleared below)
@@ -741,10 +860,11 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
             qc = A[2 * F.psum_ld];
         }
     }
-    if ((int)threadIdx.x < P.D) s_Q[threadIdx.x] = C->Q[threadIdx.x];
+    if ((int)threadIdx.x < P.D) s_Q[threadIdx.x] = PRE ? B.felt->Q[threadIdx.x] : C->Q[threadIdx.x];
     __syncthreads();
     int coll = 0;
     if (live) {
+        if (!PRE) ion_terms<CP_WIDE>(P, B, buf, i, x, y, z, cx, cy, cz, bx, by, bz);
         float ax = 0.f, ay = 0.f, az = 0.f;
         if (!(P.flags & OD_F_NO_IONION)) {
             double px = 0.0, py = 0.0, pz = 0.0;  // pair sum in scaled units
@@ -794,16 +914,6 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
                 pz = sz;
             }
             if (P.cp_on) {
-                const double* Xb = B.x[buf];
-                double cx, cy, cz;
-                close_pair_corr<CP_WIDE>(B.cp_head, B.cp_next, B.fpos, P.cp_mask, P.cp_hinv, P.cp_dc2, C->cp_epoch,
-                                         C->n_cur, P.ls_inv, i, x, y, z,
-                                         [&](int j, double& xj, double& yj, double& zj) {
-                                             xj = Xb[j];
-                                             yj = Xb[cap + j];
-                                             zj = Xb[2 * cap + j];
-                                         },
-                                         cx, cy, cz);
                 px += cx;
                 py += cy;
                 pz += cz;
@@ -823,15 +933,6 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
             ax = fmaf(c, dx, ax);
             ay = fmaf(c, dy, ay);
             az = fmaf(c, dz, az);
-        }
-        // E_out (FP64 polynomial) and the driving field
-        double bx = 0.0, by = 0.0, bz = P.qm * P.E;
-        if (P.eout) {
-            double ex, ey, ez;
-            eout_field(P, x, y, z, ex, ey, ez);
-            bx += P.qm * ex;
-            by += P.qm * ey;
-            bz += P.qm * ez;
         }
         const float4 a = make_float4((float)((double)ax + bx), (float)((double)ay + by), (float)((double)az + bz), 0.f);
         B.acc[i] = a;
@@ -870,51 +971,10 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
             F.psum[2 * F.psum_ld + e] = 0;
         }
     }
+    if (PRE) return;
     const unsigned bc = __ballot_sync(0xffffffffu, coll);
     if (lane == 0 && bc) atomicAdd(&C->ev_step[12], __popc(bc));
-
-    // grain side of Eq. 1 without the prefactor q Q_k / (4 pi eps0):
-    // sum_i (1 + rho/lambda) exp(-rho/lambda) (r_k - r_i) / rho^3; FP32 terms from FP64
-    // separations, FP64 sums in a fixed order (warp tree, then block tree)
-    const float lam_inv = (float)P.lam_inv;
-    const float lam_inv_l2 = (float)(P.lam_inv * 1.4426950408889634);
-    for (int k = 0; k < P.D; ++k) {
-        double fx = 0.0, fy = 0.0, fz = 0.0;
-        if (live) {
-            const float dx = (float)(P.gx[k] - x), dy = (float)(P.gy[k] - y), dz = (float)(P.gz[k] - z);
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float ri = rsqrt_approx(r2);
-            const float rho = r2 * ri;
-            const float f = fmaf(rho, lam_inv, 1.0f) * ex2_approx(-rho * lam_inv_l2) * (ri * ri * ri);
-            fx = (double)(f * dx);
-            fy = (double)(f * dy);
-            fz = (double)(f * dz);
-        }
-        fx = warp_sum(fx);
-        fy = warp_sum(fy);
-        fz = warp_sum(fz);
-        if (lane == 0) {
-            s_red[warp][0] = fx;
-            s_red[warp][1] = fy;
-            s_red[warp][2] = fz;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            double a0 = lane < BT / 32 ? s_red[lane][0] : 0.0;
-            double a1 = lane < BT / 32 ? s_red[lane][1] : 0.0;
-            double a2 = lane < BT / 32 ? s_red[lane][2] : 0.0;
-            a0 = warp_sum(a0);
-            a1 = warp_sum(a1);
-            a2 = warp_sum(a2);
-            if (lane == 0) {
-                double* o = B.dpart + ((long long)blk * MAXD + k) * 3;
-                o[0] = a0;
-                o[1] = a1;
-                o[2] = a2;
-            }
-        }
-        __syncthreads();
-    }
+    grain_sums<BT>(P, B, live, x, y, z, blk);
 }
 
 // --------------------------------------------------------------- grain tail

@@ -79,6 +79,13 @@ struct Rem {
     int pad;
 };
 
+// What a step's kick reads of the control block, set by the scan (the grain tail, which
+// changes the control block's, runs beside the pair forces)
+struct Felt {
+    long long step;   // steps completed before this one
+    double Q[MAXD];   // grain charges the ions feel during it
+};
+
 // Physical constants and run parameters, passed by value to every kernel.
 struct Phys {
     int N, n_pad, D, flags;  // N: ions the buffers and plans are sized for (with the flux
@@ -107,7 +114,8 @@ struct Phys {
     double e_over_kTe;
     double inv4pieps0;
     // App. B inverse flux CDFs tabulated at U = k / VTAB_K (bottom face, then top face):
-    // starting points and brackets for the Newton polish of every injected axial speed
+    // starting points and brackets for the Newton polish of every injected axial speed; then
+    // Phi(-u / sig) and phi(-u / sig)
     const double* vtab;
     double gmax_b, gmax_t;  // flux integrals G(v_max) and G_top(v_min) the CDFs are normalised by
     long long spin_limit;  // polls before a device-side wait gives up (ERR_TIMEOUT)
@@ -143,6 +151,9 @@ struct Bufs {
     Inj* inj_ahead;  // [INJ_AHEAD] injection samples of the next step, computed during this one
     double* coll_v;  // [3][cap] neutral velocities of this step's colliding ions, computed beside the
                      // pair forces (null: the kick draws them)
+    double* pre;   // [6][cap] the step's ion terms (close-pair correction, E_out and driving field),
+                   // computed beside the pair forces (single runs)
+    Felt* felt;    // null in a batch
     double* dpart; // grain partial sums [nb][MAXD][3]
     Ctrl* ctrl;
     long long cap;
@@ -208,10 +219,14 @@ int launch_push_scan(const Phys& P, const Bufs& B, cudaStream_t s);
 int launch_forces(const Phys& P, const Bufs& B, const ForceArgs& F, int variant, cudaStream_t s);
 int launch_kick(const Phys& P, const Bufs& B, const ForceArgs& F, int mode, cudaStream_t s);
 int launch_cp_bump(const Bufs& B, cudaStream_t s);  // advance the close-pair list epoch
-// the next step's first INJ_AHEAD injection samples (run beside the pair forces)
+int launch_kick_step(const Phys& P, const Bufs& B, const ForceArgs& F, cudaStream_t s);
+// beside a step's pair forces: the next step's first INJ_AHEAD injection samples, the ion
+// terms and collision velocities its kick adds (Bufs::pre, coll_v), and the grain side
+// (Eq. 1 sums, then the grain tail)
 int launch_inject_ahead(const Phys& P, const Bufs& B, cudaStream_t s);
-// this step's collision velocities (Bufs::coll_v), beside the pair forces
-int launch_collide_ahead(const Phys& P, const Bufs& B, cudaStream_t s);
+int launch_ion_terms(const Phys& P, const Bufs& B, cudaStream_t s);
+int launch_grains(const Phys& P, const Bufs& B, cudaStream_t s);
+int launch_vtab_consts(double* vtab, double u, double sig, cudaStream_t s);
 // OML floating charge of every grain into Ctrl::Q (nq Gauss-Legendre nodes glx, glw on [-1, 1])
 // E_out at the grain centres into Ctrl::eg (once, at creation)
 int launch_grain_eout(const Phys& P, const Bufs& B, cudaStream_t s);

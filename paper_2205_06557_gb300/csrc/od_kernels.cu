@@ -1,14 +1,22 @@
 // CUDA kernels of the ion-flow-around-dust step for GB300 (sm_103a).
 //
-// One time step is four kernels, in the canonical order of the method (Sec. 2):
+// One time step, in the canonical order of the method (Sec. 2):
 //   k_push_scan  first half kick + drift (velocity Verlet), absorption / outflow test,
 //                single-pass decoupled-look-back scan of the removal flags, stable
 //                compaction into the other state buffer, and 1:1 re-injection (App. B)
-//   k_forces     all-pairs Yukawa ion-ion forces in FP32 (persistent, balanced tiles)
-//   k_kick       grain Coulomb force, E_out (App. A) and E_ext on ions, second half kick,
-//                Andersen collisions, and the grain-side Yukawa sums of Eq. 1 (FP64); its
-//                last block runs the grain tail: Eq. 1-4 terms, charge update, records,
-//                time averages
+//   k_forces*    all-pairs Yukawa ion-ion forces in FP32; beside them, on three more streams:
+//                  k_ion_terms     close-pair correction, E_out (App. A) and E_ext on the ions,
+//                                  collision velocities
+//                  k_grains        the grain-side Yukawa sums of Eq. 1 (FP64); its last block runs
+//                                  the grain tail: Eq. 1-4 terms, charge update, records,
+//                                  time averages
+//                  k_inject_ahead  the next step's injection samples
+//   k_kick_step  pair forces, ion terms and grain Coulomb force on ions, second half kick,
+//                Andersen collisions
+// A run of a few thousand ions is bound by the latency of this chain (FP64 dependencies and
+// memory round trips), which is why what does not need the pair forces runs beside them
+// (~2,000 ions: 47.2 us per step with all of it in the kick, 34.3 us beside the pair forces;
+// 35,000 ions under the flux rule 486 -> 466 us).
 // Every kernel reads the step number from device memory, so a captured graph of one
 // step replays without the host.
 #include <algorithm>
@@ -70,20 +78,44 @@ __global__ void k_init_ions(Phys P, Bufs B, double ls_inv)
 // for step ahead_req_sn, all set by this step's scan), launched on a second stream beside
 // the pair forces; the next scan uses them where the tag matches and draws the rest
 // itself.  The tag is written after the samples.
-constexpr int INJ_BT = 32;  // one warp per block: FP64 is slow on this GPU, so the draws
-                            // are spread over as many SMs as there are warps of them
+// Latency bound (FP64 is slow on this GPU and a sample is ~20 us of dependent FP64 in one
+// thread): a block of four warps draws 32 samples, one independent part of every sample per warp
+// (normals, angle, axial speed, radial speed), and the first warp puts them together.
+constexpr int INJ_SAMPLES = 32, INJ_BT = 4 * INJ_SAMPLES;
 
 __global__ void __launch_bounds__(INJ_BT) k_inject_ahead(Phys P, Bufs B)
 {
     __shared__ int s_last;
+    __shared__ double s_s[INJ_SAMPLES], s_c[INJ_SAMPLES], s_ax[INJ_SAMPLES], s_rad[INJ_SAMPLES];
     Ctrl* C = B.ctrl;
     const long long sn = C->ahead_req_sn;
     const unsigned long long base = C->next_id;
-    const int want = min(C->ahead_want, (int)(gridDim.x * INJ_BT));
-    const int r = blockIdx.x * INJ_BT + threadIdx.x;
-    if (sn > 0 && r < want) {
+    const int want = min(C->ahead_want, (int)(gridDim.x * INJ_SAMPLES));
+    const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+    const int r = blockIdx.x * INJ_SAMPLES + lane;
+    const bool draw = sn > 0 && r < want;
+    uint4 A = make_uint4(0u, 0u, 0u, 0u);
+    int face = 0;
+    double n0 = 0.0, n1 = 0.0;
+    if (draw) {
+        A = philox(P, base + (unsigned long long)r, (uint32_t)sn, ST_INJ_A);
+        face = inj_face(P, A);
+        if (part == 0) {
+            const uint4 Bw = philox(P, base + (unsigned long long)r, (uint32_t)sn, ST_INJ_B);
+            box_muller(Bw.x, Bw.y, n0, n1);
+        } else if (part == 1) {
+            inj_angle(face, A, s_s[lane], s_c[lane]);
+        } else if (part == 2) {
+            if (face != 2) s_ax[lane] = inj_axial(P, face, A);
+        } else if (face == 2) {
+            s_rad[lane] = inj_radial(P, A);
+        }
+    }
+    __syncthreads();
+    if (draw && part == 0) {
         Inj o;
-        sample_injection(P, base + (unsigned long long)r, (uint32_t)sn, o);
+        inj_assemble(P, base + (unsigned long long)r, face, A, n0, n1, s_s[lane], s_c[lane],
+                     face == 2 ? s_rad[lane] : s_ax[lane], o);
         o.pad = 0;
         B.inj_ahead[r] = o;
     }
@@ -102,38 +134,99 @@ __global__ void __launch_bounds__(INJ_BT) k_inject_ahead(Phys P, Bufs B)
     }
 }
 
-// This step's collision velocities, beside the pair forces: the ions' order and ids are
-// final after the scan, and a collision depends only on (seed, id, step), so the kick
-// finds the FP64 Box-Muller draws of its colliding ions ready.
-__global__ void k_collide_ahead(Phys P, Bufs B)
+// What this step's kick adds besides the pair forces, beside them: the ions' order and
+// positions are final after the scan.  Close-pair correction, E_out and the driving field of
+// every ion, and the FP64 Box-Muller draws of the colliding ones (a collision depends only
+// on (seed, id, step)).
+__global__ void __launch_bounds__(KICK_BT) k_ion_terms(Phys P, Bufs B)
 {
     const Ctrl* C = B.ctrl;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * KICK_BT + threadIdx.x;
     if (i >= C->n_cur) return;
-    const long long step = C->step;
+    const long long step = B.felt->step, cap = B.cap;
     const int buf = (int)((step + 1) & 1);
     const uint32_t sn = (uint32_t)(step + 1);
+    const double* X = B.x[buf];
+    const double x = X[i], y = X[cap + i], z = X[2 * cap + i];
     const unsigned long long id = B.id[buf][i];
+    double cx, cy, cz, bx, by, bz;
+    ion_terms<8>(P, B, buf, i, x, y, z, cx, cy, cz, bx, by, bz);
+    double* T = B.pre;
+    T[i] = cx, T[cap + i] = cy, T[2 * cap + i] = cz;
+    T[3 * cap + i] = bx, T[4 * cap + i] = by, T[5 * cap + i] = bz;
     const uint4 w = philox(P, id, sn, ST_COLL);
     if ((unsigned long long)w.x >= P.Tcoll) return;
     double vx, vy, vz;
     collision_velocity(P, id, sn, vx, vy, vz);
     B.coll_v[i] = vx;
-    B.coll_v[B.cap + i] = vy;
-    B.coll_v[2 * B.cap + i] = vz;
+    B.coll_v[cap + i] = vy;
+    B.coll_v[2 * cap + i] = vz;
 }
 
-int launch_collide_ahead(const Phys& P, const Bufs& B, cudaStream_t s)
+int launch_ion_terms(const Phys& P, const Bufs& B, cudaStream_t s)
 {
-    if (P.N == 0 || !B.coll_v) return 0;
-    k_collide_ahead<<<(P.N + 255) / 256, 256, 0, s>>>(P, B);
+    if (P.N == 0) return 0;
+    k_ion_terms<<<(P.N + KICK_BT - 1) / KICK_BT, KICK_BT, 0, s>>>(P, B);
+    return (int)cudaGetLastError();
+}
+
+// The grain side of a step, beside the pair forces: it needs the ions' positions, the
+// charges and the events, none of which the pair forces or the kick change.  Eq. 1 sums and
+// collision counts, then the grain tail in the last block to finish.
+__global__ void __launch_bounds__(KICK_BT) k_grains(Phys P, Bufs B)
+{
+    __shared__ int s_last;
+    Ctrl* C = B.ctrl;
+    const int i = blockIdx.x * KICK_BT + threadIdx.x;
+    const bool live = i < C->n_cur;
+    const long long step = B.felt->step, cap = B.cap;
+    const int buf = (int)((step + 1) & 1);
+    double x = 0, y = 0, z = 0;
+    int coll = 0;
+    if (live) {
+        const double* X = B.x[buf];
+        x = X[i], y = X[cap + i], z = X[2 * cap + i];
+        const uint4 w = philox(P, B.id[buf][i], (uint32_t)(step + 1), ST_COLL);
+        coll = (unsigned long long)w.x < P.Tcoll;
+    }
+    const unsigned bc = __ballot_sync(0xffffffffu, coll);
+    if ((threadIdx.x & 31) == 0 && bc) atomicAdd(&C->ev_step[12], __popc(bc));
+    grain_sums<KICK_BT>(P, B, live, x, y, z, blockIdx.x);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&C->kick_done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) C->kick_done = 0u;
+    dust_body(P, B, (int)gridDim.x, 0);
+}
+
+int launch_grains(const Phys& P, const Bufs& B, cudaStream_t s)
+{
+    if (P.N == 0) return 0;
+    k_grains<<<(P.N + KICK_BT - 1) / KICK_BT, KICK_BT, 0, s>>>(P, B);
+    return (int)cudaGetLastError();
+}
+
+// Phi(z0) and phi(z0), z0 = -u / sig, after the tabulated inverse flux CDFs
+__global__ void k_vtab_consts(double* vtab, double u, double sig)
+{
+    const double z0 = -u / sig;
+    vtab[2 * (VTAB_K + 1)] = ncdf(z0);
+    vtab[2 * (VTAB_K + 1) + 1] = npdf(z0);
+}
+
+int launch_vtab_consts(double* vtab, double u, double sig, cudaStream_t s)
+{
+    k_vtab_consts<<<1, 1, 0, s>>>(vtab, u, sig);
     return (int)cudaGetLastError();
 }
 
 int launch_inject_ahead(const Phys& P, const Bufs& B, cudaStream_t s)
 {
     if (P.N == 0) return 0;
-    k_inject_ahead<<<INJ_AHEAD / INJ_BT, INJ_BT, 0, s>>>(P, B);
+    k_inject_ahead<<<INJ_AHEAD / INJ_SAMPLES, INJ_BT, 0, s>>>(P, B);
     return (int)cudaGetLastError();
 }
 
@@ -183,8 +276,14 @@ __global__ void __launch_bounds__(BT) k_push_scan(Phys P, Bufs B, int n_tiles, d
     push_scan_body<BT>(P, B, n_tiles, ls_inv, -1);
 }
 
-// The kick, then the grain tail in the last block to finish (the grain update reads every
-// block's sums; one launch fewer per step than a separate tail kernel)
+// A step's kick: the pair forces, the precomputed ion terms and the grain Coulomb force
+__global__ void __launch_bounds__(KICK_BT) k_kick_step(Phys P, Bufs B, ForceArgs F)
+{
+    kick_body<KICK_BT, 8, true>(P, B, F, 0, blockIdx.x);
+}
+
+// The whole kick, then the grain tail in the last block to finish (the grain update reads every
+// block's sums): force evaluations outside the steps
 template <int BT>
 __global__ void __launch_bounds__(BT) k_kick(Phys P, Bufs B, ForceArgs F, int mode)
 {
@@ -472,7 +571,7 @@ constexpr int F64_BT = 128;
 __global__ void __launch_bounds__(F64_BT) k_forces_f64(Phys P, Bufs B, int after_push, double ls_inv)
 {
     __shared__ double sx[F64_BT], sy[F64_BT], sz[F64_BT];
-    const long long step = B.ctrl->step;
+    const long long step = after_push ? B.felt->step : B.ctrl->step;
     const int buf = after_push ? (int)((step + 1) & 1) : (int)(step & 1);
     const double* X = B.x[buf];
     const int n = B.ctrl->n_cur;
@@ -547,6 +646,13 @@ int launch_kick(const Phys& P, const Bufs& B, const ForceArgs& F, int mode, cuda
     return ck(cudaGetLastError());
 }
 
+
+int launch_kick_step(const Phys& P, const Bufs& B, const ForceArgs& F, cudaStream_t s)
+{
+    if (P.N == 0) return 0;
+    k_kick_step<<<(P.N + KICK_BT - 1) / KICK_BT, KICK_BT, 0, s>>>(P, B, F);
+    return ck(cudaGetLastError());
+}
 
 // host interface layouts: the ABI's interleaved [n][3] arrays <-> the device's [3][cap]
 // structure of arrays (and the float4 accelerations), converted on the device so that a
