@@ -802,7 +802,7 @@ int create_impl(const od_params* p, od_handle* h)
     {
         std::vector<double> tab;
         build_vtab(h->P.u, h->P.sig, tab, h->P.gmax_b, h->P.gmax_t);
-        OD_CK(h, cudaMalloc(&h->d_vtab, sizeof(double) * (tab.size() + 2)));
+        OD_CK(h, cudaMalloc(&h->d_vtab, sizeof(double) * (tab.size() + 3)));
         OD_CK(h, cudaMemcpyAsync(h->d_vtab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice, h->stream));
         OD_LK(h, launch_vtab_consts(h->d_vtab, h->P.u, h->P.sig, h->stream));
         OD_CK(h, cudaStreamSynchronize(h->stream));
@@ -850,8 +850,9 @@ int create_impl(const od_params* p, od_handle* h)
     OD_CK(h, cudaMalloc(&B.cp_head, sizeof(unsigned long long) * nbk));
     OD_CK(h, cudaMemsetAsync(B.cp_head, 0, sizeof(unsigned long long) * nbk, h->stream));
     OD_CK(h, cudaMalloc(&B.cp_next, sizeof(int) * h->cap));
-    // one status word per scan tile: single runs scan 256-ion tiles, batch members 128
-    const long long scan_tile = std::min(push_tile(), BATCH_TILE);
+    // one status word per scan tile: single runs scan 256- or 64-ion tiles (the fewer ions of a
+    // replaced state may take the small ones), batch members 128
+    const long long scan_tile = std::min(push_tile(0), BATCH_TILE);
     const long long ntiles = (h->cap + scan_tile - 1) / scan_tile;
     h->scan_tiles_cap = ntiles;
     OD_CK(h, cudaMalloc(&B.tile_status, sizeof(unsigned long long) * ntiles));
@@ -1258,7 +1259,7 @@ int od_oml_charge(const od_params* p, double radius, double* Q)
 int od_selftest_wait_timeout(od_handle* h, int64_t polls)
 {
     if (!h || polls < 1) return fail(h, OD_EINVAL, "bad handle or poll limit");
-    if (h->P.N <= push_tile()) return fail(h, OD_EINVAL, "the wait self-test needs more than one scan tile");
+    if (h->P.N <= 256) return fail(h, OD_EINVAL, "the wait self-test needs more than one scan tile");
     Phys P = h->P;
     P.spin_limit = polls;
     P.test_hold_tile0 = 1;

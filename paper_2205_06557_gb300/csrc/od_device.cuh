@@ -54,38 +54,40 @@ __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, double& n0, d
 __device__ __forceinline__ double ncdf(double z) { return 0.5 * erfc(-z * 0.70710678118654752); }
 __device__ __forceinline__ double npdf(double z) { return exp(-0.5 * z * z) * 0.39894228040143268; }
 
-// Invert a monotone App. B flux CDF on [lo, hi] for the value target: Newton steps with
-// derivative |v| N(v; u, s^2), kept inside a shrinking bracket (bisection when a step
-// leaves it).  The bottom face's flux up to axial speed v is
+// Invert a monotone App. B flux CDF on [lo, hi] for the value target: Halley steps (cubic
+// convergence: FP64 evaluations are ~4 us of latency each on this GPU, and most samples
+// need one), kept inside a shrinking bracket (bisection when a step leaves it).  The bottom
+// face's flux up to axial speed v is
 //   int_0^v v' N(v'; u, s^2) dv' = u (Phi(z) - Phi(z0)) + s (phi(z0) - phi(z)),
 // the top face's from v < 0 up to 0 is the same expression, decreasing in v, with
-// z = (v - u) / s, z0 = -u / s (Phi, phi the standard normal CDF and density; c0 = Phi(z0)
-// and p0 = phi(z0) are the run's constants).
+// z = (v - u) / s, z0 = -u / s (Phi, phi the standard normal CDF and density; c0 = Phi(z0),
+// p0 = phi(z0) and s_inv = 1 / s are the run's constants).  Its first derivative is
+// v phi(z) / s, and the ratio of the second to the first q = 1 / v - z / s.
 static __device__ double invert_flux(bool top, double target, double lo, double hi, double v, double u, double s,
-                                     double c0, double p0)
+                                     double s_inv, double c0, double p0)
 {
     for (int it = 0; it < 100; ++it) {
-        const double z = (v - u) / s;
+        const double z = (v - u) * s_inv;
         const double cz = ncdf(z), pz = npdf(z);
         const double F = u * (cz - c0) + s * (p0 - pz);
         const double g = top ? (target - F) : (F - target);  // increasing in v
         if (g < 0) lo = v;
         else hi = v;
-        const double dg = fabs(v) * pz / s;
-        // converged once the Newton correction is below ~1e-13 of the speed scale; the
-        // check comes before the bracket test, which a sub-ulp step would fail
-        const double tol = 1e-13 * fmax(fabs(v), s);
-        if (dg > 0) {
-            const double step = g / dg;
-            if (fabs(step) <= tol) {
-                v -= step;
-                break;
+        const double w = fabs(v) * pz;  // s times the derivative
+        double vn = 0.5 * (lo + hi);
+        if (w > 0) {
+            const double r = 1.0 / w;
+            const double st = g * s * r, h = 0.5 * st * (copysign(r * pz, v) - z * s_inv);
+            if (fabs(h) < 0.5) {
+                const double vh = v - (fabs(h) < 1e-5 ? st * (1.0 + h * (1.0 + h)) : st / (1.0 - h));
+                // converged: what this step leaves, ~|st|^3 q^2, is below 1e-15 of the speed
+                // scale (checked before the bracket test, which a sub-ulp step would fail)
+                if (fabs(st) < 1e-5 * s && fabs(h) < 1e-5) return vh;
+                if (vh > lo && vh < hi) vn = vh;
             }
         }
-        double vn = dg > 0 ? v - g / dg : 0.5 * (lo + hi);
-        if (!(vn > lo && vn < hi)) vn = 0.5 * (lo + hi);
         v = vn;
-        if (hi - lo <= tol) break;
+        if (hi - lo <= 1e-13 * fmax(fabs(v), s)) break;
     }
     return v;
 }
@@ -115,13 +117,13 @@ __device__ __forceinline__ double inj_axial(const Phys& P, int face, uint4 A)
     const int k = min((int)xk, VTAB_K - 1);
     const double* tab = P.vtab + (face == 0 ? 0 : VTAB_K + 1);
     const double t0 = tab[k], t1 = tab[k + 1];
-    const double c0 = P.vtab[2 * (VTAB_K + 1)], p0 = P.vtab[2 * (VTAB_K + 1) + 1];
+    const double *cst = P.vtab + 2 * (VTAB_K + 1), c0 = cst[0], p0 = cst[1], s_inv = cst[2];
     const double pad = 1e-12 * fmax(fmax(fabs(t0), fabs(t1)), P.sig);
     const double v0 = t0 + (xk - k) * (t1 - t0);
     double lo = fmin(t0, t1) - pad, hi = fmax(t0, t1) + pad;
     if (face == 0) lo = fmax(lo, 0.0);
     else hi = fmin(hi, 0.0);
-    return invert_flux(face == 1, U * (face == 0 ? P.gmax_b : P.gmax_t), lo, hi, v0, P.u, P.sig, c0, p0);
+    return invert_flux(face == 1, U * (face == 0 ? P.gmax_b : P.gmax_t), lo, hi, v0, P.u, P.sig, s_inv, c0, p0);
 }
 
 // flux-weighted radial speed through the side (Rayleigh)
@@ -164,21 +166,20 @@ static __device__ void sample_injection(const Phys& P, unsigned long long id, ui
     inj_assemble(P, id, face, A, n0, n1, s, c, sp, o);
 }
 
-// The App. B sample of the ion with this id entering in step sn: computed ahead (during
+// The App. B sample of the r-th ion entering in step sn (id base + r): computed ahead (during
 // the previous step, beside the pair forces) when it is there, else now.  A sample is a
 // function of (seed, id, sn) and the run's constants only, so both give the same bits.
-static __device__ __forceinline__ void injection_for(const Phys& P, const Bufs& B, const Ctrl* C,
-                                                     unsigned long long base, int r, uint32_t sn, Inj& o)
+__device__ __forceinline__ bool injection_ahead(const Ctrl* C, unsigned long long base, int r, uint32_t sn)
 {
-    if (r < C->ahead_n && C->ahead_base == base && C->ahead_sn == (long long)sn) {
-        const Inj* a = B.inj_ahead + r;
-        o.x = __ldcg(&a->x), o.y = __ldcg(&a->y), o.z = __ldcg(&a->z);
-        o.vx = __ldcg(&a->vx), o.vy = __ldcg(&a->vy), o.vz = __ldcg(&a->vz);
-        o.id = __ldcg(&a->id);
-        o.face = __ldcg(&a->face);
-    } else {
-        sample_injection(P, base + (unsigned long long)r, sn, o);
-    }
+    return r < C->ahead_n && C->ahead_base == base && C->ahead_sn == (long long)sn;
+}
+
+__device__ __forceinline__ void load_injection(const Inj* a, Inj& o)
+{
+    o.x = __ldcg(&a->x), o.y = __ldcg(&a->y), o.z = __ldcg(&a->z);
+    o.vx = __ldcg(&a->vx), o.vy = __ldcg(&a->vy), o.vz = __ldcg(&a->vz);
+    o.id = __ldcg(&a->id);
+    o.face = __ldcg(&a->face);
 }
 
 // Andersen collision: a zero-mean Maxwellian velocity at the neutral temperature
@@ -429,7 +430,8 @@ __device__ __forceinline__ int poisson_injections(const Phys& P, uint32_t sn)
 }
 
 // ------------------------------------------------- push + scan + compaction
-constexpr int PUSH_BT = 256;
+constexpr int PUSH_BT = 256;       // ions per scan tile of a single run
+constexpr int PUSH_BT_SMALL = 64;  // and of one small enough for a tile per SM (FP64 is slow)
 
 constexpr unsigned FLAG_A = 1u, FLAG_P = 2u;
 
@@ -614,13 +616,11 @@ __device__ __forceinline__ void push_scan_body(const Phys& P, const Bufs& B, int
             rm.cls = cls;
             rm.pad = 0;
             B.rem[r] = rm;
-            if (!flux) {  // 1:1 replacement: the removed ion's thread samples its successor
+            if (!flux && !injection_ahead(C, C->next_id, r, sn)) {
+                // 1:1 replacement beyond the samples drawn ahead: the removed ion's thread
+                // samples its successor
                 Inj in;
-                injection_for(P, B, C, C->next_id, r, sn, in);
-                if (P.flags & OD_F_FP32_STATE) {
-                    in.x = rnd32(in.x), in.y = rnd32(in.y), in.z = rnd32(in.z);
-                    in.vx = rnd32(in.vx), in.vy = rnd32(in.vy), in.vz = rnd32(in.vz);
-                }
+                sample_injection(P, C->next_id + (unsigned long long)r, sn, in);
                 in.pad = 0;
                 B.inj[r] = in;
             }
@@ -651,38 +651,28 @@ __device__ __forceinline__ void push_scan_body(const Phys& P, const Bufs& B, int
     __syncthreads();
     const int m = s_m, kin = s_k;
     for (int r = threadIdx.x; r < kin; r += BT) {
-        double ix, iy, iz, ivx, ivy, ivz;
-        unsigned long long iid;
-        int face;
-        if (flux) {
-            Inj in;
-            injection_for(P, B, C, C->next_id, r, sn, in);
-            if (P.flags & OD_F_FP32_STATE) {
-                in.x = rnd32(in.x), in.y = rnd32(in.y), in.z = rnd32(in.z);
-                in.vx = rnd32(in.vx), in.vy = rnd32(in.vy), in.vz = rnd32(in.vz);
-            }
-            ix = in.x, iy = in.y, iz = in.z, ivx = in.vx, ivy = in.vy, ivz = in.vz, iid = in.id, face = in.face;
-        } else {
-            const Inj* in = B.inj + r;
-            ix = __ldcg(&in->x), iy = __ldcg(&in->y), iz = __ldcg(&in->z);
-            ivx = __ldcg(&in->vx), ivy = __ldcg(&in->vy), ivz = __ldcg(&in->vz);
-            iid = __ldcg(&in->id);
-            face = __ldcg(&in->face);
+        Inj in;
+        if (injection_ahead(C, C->next_id, r, sn)) load_injection(B.inj_ahead + r, in);
+        else if (!flux) load_injection(B.inj + r, in);
+        else sample_injection(P, C->next_id + (unsigned long long)r, sn, in);
+        if (P.flags & OD_F_FP32_STATE) {
+            in.x = rnd32(in.x), in.y = rnd32(in.y), in.z = rnd32(in.z);
+            in.vx = rnd32(in.vx), in.vy = rnd32(in.vy), in.vz = rnd32(in.vz);
         }
         const int d = n_live - m + r;
         double* X = B.x[dst];
         double* V = B.v[dst];
-        X[d] = ix;
-        X[cap + d] = iy;
-        X[2 * cap + d] = iz;
-        V[d] = ivx;
-        V[cap + d] = ivy;
-        V[2 * cap + d] = ivz;
-        B.id[dst][d] = iid;
-        const float4 f = scaled(P, ix, iy, iz, ls_inv);
+        X[d] = in.x;
+        X[cap + d] = in.y;
+        X[2 * cap + d] = in.z;
+        V[d] = in.vx;
+        V[cap + d] = in.vy;
+        V[2 * cap + d] = in.vz;
+        B.id[dst][d] = in.id;
+        const float4 f = scaled(P, in.x, in.y, in.z, ls_inv);
         B.fpos[d] = f;
         if (P.cp_on) cp_insert(B.cp_head, B.cp_next, P.cp_mask, P.cp_hinv, cp_ep, d, f);
-        atomicAdd(&s_face[face], 1);
+        atomicAdd(&s_face[in.face], 1);
     }
     // slots vacated when fewer ions entered than left: far-away dummies for the pair kernel
     const int n_new = n_live - m + kin;
@@ -730,26 +720,27 @@ __device__ __forceinline__ double warp_sum(double v)
 }
 
 // What a step's kick adds that does not depend on the pair forces, for ion i at (x, y, z):
-// the close-pair correction (scaled units) and the acceleration of E_out (FP64 polynomial)
-// and the driving field.
+// the close-pair correction (scaled units) ...
 template <int CP_WIDE>
-__device__ __forceinline__ void ion_terms(const Phys& P, const Bufs& B, int buf, int i, double x, double y, double z,
-                                          double& cx, double& cy, double& cz, double& bx, double& by, double& bz)
+__device__ __forceinline__ void close_pairs_of(const Phys& P, const Bufs& B, int buf, int i, double x, double y,
+                                               double z, double& cx, double& cy, double& cz)
 {
     const Ctrl* C = B.ctrl;
-    cx = cy = cz = 0.0;
-    if (P.cp_on) {
-        const double* Xb = B.x[buf];
-        const long long cap = B.cap;
-        close_pair_corr<CP_WIDE>(B.cp_head, B.cp_next, B.fpos, P.cp_mask, P.cp_hinv, P.cp_dc2, C->cp_epoch, C->n_cur,
-                                 P.ls_inv, i, x, y, z,
-                                 [&](int j, double& xj, double& yj, double& zj) {
-                                     xj = Xb[j];
-                                     yj = Xb[cap + j];
-                                     zj = Xb[2 * cap + j];
-                                 },
-                                 cx, cy, cz);
-    }
+    const double* Xb = B.x[buf];
+    const long long cap = B.cap;
+    close_pair_corr<CP_WIDE>(B.cp_head, B.cp_next, B.fpos, P.cp_mask, P.cp_hinv, P.cp_dc2, C->cp_epoch, C->n_cur,
+                             P.ls_inv, i, x, y, z,
+                             [&](int j, double& xj, double& yj, double& zj) {
+                                 xj = Xb[j];
+                                 yj = Xb[cap + j];
+                                 zj = Xb[2 * cap + j];
+                             },
+                             cx, cy, cz);
+}
+
+// ... and the acceleration of E_out (FP64 polynomial) and the driving field
+__device__ __forceinline__ void ion_field(const Phys& P, double x, double y, double z, double& bx, double& by, double& bz)
+{
     bx = by = 0.0;
     bz = P.qm * P.E;
     if (P.eout) {
@@ -864,7 +855,8 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
     __syncthreads();
     int coll = 0;
     if (live) {
-        if (!PRE) ion_terms<CP_WIDE>(P, B, buf, i, x, y, z, cx, cy, cz, bx, by, bz);
+        if (!PRE && P.cp_on) close_pairs_of<CP_WIDE>(P, B, buf, i, x, y, z, cx, cy, cz);
+        if (!PRE) ion_field(P, x, y, z, bx, by, bz);
         float ax = 0.f, ay = 0.f, az = 0.f;
         if (!(P.flags & OD_F_NO_IONION)) {
             double px = 0.0, py = 0.0, pz = 0.0;  // pair sum in scaled units
@@ -989,7 +981,7 @@ __device__ __forceinline__ void dust_body(const Phys& P, const Bufs& B, int nb, 
     __shared__ double s_S[MAXD][3];
     __shared__ double s_pm[MAXD][3];
     __shared__ double s_rec[MAXD][REC];
-    __shared__ double s_Qd[MAXD];
+    __shared__ double s_Qd[MAXD], s_Qn[MAXD];
     Ctrl* C = B.ctrl;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
     const int k = threadIdx.x, j = threadIdx.x;
@@ -1002,10 +994,8 @@ __device__ __forceinline__ void dust_body(const Phys& P, const Bufs& B, int nb, 
     double* const series = C->series;
     int* const evseries = C->evseries;
     double Qk = 0.0, wk[REC], egx = 0.0, egy = 0.0, egz = 0.0;
-    int evk = 0;
     if (k < P.D) {
         Qk = C->Q[k];
-        evk = C->ev_step[k];
         egx = C->eg[k][0];
         egy = C->eg[k][1];
         egz = C->eg[k][2];
@@ -1047,11 +1037,26 @@ __device__ __forceinline__ void dust_body(const Phys& P, const Bufs& B, int nb, 
         px = warp_sum(px);
         py = warp_sum(py);
         pz = warp_sum(pz);
-        if (lane == 0) {
-            s_pm[kk][0] = P.m * px;
-            s_pm[kk][1] = P.m * py;
-            s_pm[kk][2] = P.m * pz;
+        px = __shfl_sync(0xffffffffu, px, 0);
+        py = __shfl_sync(0xffffffffu, py, 0);
+        pz = __shfl_sync(0xffffffffu, pz, 0);
+        if (lane < 3) s_pm[kk][lane] = P.m * (lane == 0 ? px : lane == 1 ? py : pz) / P.dt;
+    }
+    // the charge update (explicit: the forces use the charge before it), of grain k in the last
+    // warp, beside the sums of the others
+    const int ku = (int)threadIdx.x - 32 * (nw - 1);
+    if (mode == 0 && ku >= 0 && ku < P.D) {
+        const double Q = C->Q[ku];
+        double Qn = Q;
+        if (P.charge_model == OD_Q_CONSISTENT) {
+            // absorbed superions plus the OML electron flux at the isolated-sphere potential
+            const double a = P.ga[ku];
+            const double xe = Q * P.inv4pieps0 / a * P.e_over_kTe;
+            const double fac = xe <= 0.0 ? exp(xe) : 1.0 + xe;
+            const double flux = 4.0 * 3.141592653589793 * a * a * P.Ie0 * fac;
+            Qn = Q + P.q * (double)C->ev_step[ku] - 1.602176634e-19 * flux * P.dt;
         }
+        s_Qn[ku] = Qn;
     }
     if (k < P.D) s_Qd[k] = Qk;
     __syncthreads();
@@ -1076,22 +1081,13 @@ __device__ __forceinline__ void dust_body(const Phys& P, const Bufs& B, int nb, 
             for (int t = 0; t < 3; ++t) {
                 s_rec[k][1 + t] = fo[t];
                 s_rec[k][4 + t] = fdd[t];
-                s_rec[k][7 + t] = s_pm[k][t] / P.dt;
+                s_rec[k][7 + t] = s_pm[k][t];
             }
             s_rec[k][10] = 0.0;
             s_rec[k][11] = 0.0;
             s_rec[k][12] = Q * P.E;  // Eq. 4
-            // the charge update (explicit: the forces above used the charge before it)
-            double Qn = Q;
-            if (P.charge_model == OD_Q_CONSISTENT) {
-                // absorbed superions plus the OML electron flux at the isolated-sphere potential
-                const double a = P.ga[k];
-                const double xe = Q * P.inv4pieps0 / a * P.e_over_kTe;
-                const double fac = xe <= 0.0 ? exp(xe) : 1.0 + xe;
-                const double flux = 4.0 * 3.141592653589793 * a * a * P.Ie0 * fac;
-                Qn = Q + P.q * (double)evk - 1.602176634e-19 * flux * P.dt;
-                C->Q[k] = Qn;
-            }
+            const double Qn = s_Qn[k];
+            if (P.charge_model == OD_Q_CONSISTENT) C->Q[k] = Qn;
             s_rec[k][0] = Qn;
             if (step < scap) {
                 double* o = series + (step * MAXD + k) * REC;
@@ -1102,8 +1098,8 @@ __device__ __forceinline__ void dust_body(const Phys& P, const Bufs& B, int nb, 
         }
     }
     if (mode != 0) return;
-    // one thread per event counter: record, accumulate, reset for the next step (the grain
-    // threads above read their own counts before this block reaches here: the barrier)
+    // one thread per event counter: record, accumulate, reset for the next step (the charge
+    // update above has read the counts: the barriers)
     __syncthreads();
     const long long sn = step + 1;
     if (j < EV) {

@@ -115,7 +115,7 @@ struct Phys {
     double inv4pieps0;
     // App. B inverse flux CDFs tabulated at U = k / VTAB_K (bottom face, then top face):
     // starting points and brackets for the Newton polish of every injected axial speed; then
-    // Phi(-u / sig) and phi(-u / sig)
+    // Phi(-u / sig), phi(-u / sig) and 1 / sig
     const double* vtab;
     double gmax_b, gmax_t;  // flux integrals G(v_max) and G_top(v_min) the CDFs are normalised by
     long long spin_limit;  // polls before a device-side wait gives up (ERR_TIMEOUT)
@@ -276,7 +276,8 @@ int force_blocks_per_sm(int variant);
 // message returned by od_last_error(NULL) for calls without a handle (od_api.cu)
 void set_global_error(const std::string& msg);
 
-int push_tile();  // ions per scan tile
+constexpr int PUSH_SMALL_MAX = 64 * 152;  // ions up to which the scan takes its small tiles
+int push_tile(int N);  // ions per scan tile
 int kick_block(); // threads per block of the kick kernel
 
 }  // namespace od

@@ -15,8 +15,9 @@
 //                Andersen collisions
 // A run of a few thousand ions is bound by the latency of this chain (FP64 dependencies and
 // memory round trips), which is why what does not need the pair forces runs beside them
-// (~2,000 ions: 47.2 us per step with all of it in the kick, 34.3 us beside the pair forces;
-// 35,000 ions under the flux rule 486 -> 466 us).
+// (~2,000 ions, from scan to scan: 45.9 us with all of it in the kick, ~33 us beside the pair
+// forces, 27.7 us with the samples drawn by parts and mostly one FP64 evaluation, the ion
+// terms in one-warp blocks per chain, and the injected ions placed straight from the samples).
 // Every kernel reads the step number from device memory, so a captured graph of one
 // step replays without the host.
 #include <algorithm>
@@ -135,38 +136,50 @@ __global__ void __launch_bounds__(INJ_BT) k_inject_ahead(Phys P, Bufs B)
 }
 
 // What this step's kick adds besides the pair forces, beside them: the ions' order and
-// positions are final after the scan.  Close-pair correction, E_out and the driving field of
-// every ion, and the FP64 Box-Muller draws of the colliding ones (a collision depends only
+// positions are final after the scan.  Three independent chains per ion, each of FP64
+// dependencies and memory round trips, in blocks of their own (blockIdx.y) of one warp, so
+// that they run at the same time on different SMs: the close-pair correction; E_out and the
+// driving field; the FP64 Box-Muller draws of the colliding ions (a collision depends only
 // on (seed, id, step)).
-__global__ void __launch_bounds__(KICK_BT) k_ion_terms(Phys P, Bufs B)
+constexpr int TERMS_BT = 32;
+
+__global__ void __launch_bounds__(TERMS_BT) k_ion_terms(Phys P, Bufs B)
 {
     const Ctrl* C = B.ctrl;
-    const int i = blockIdx.x * KICK_BT + threadIdx.x;
+    const int i = blockIdx.x * TERMS_BT + threadIdx.x;
     if (i >= C->n_cur) return;
     const long long step = B.felt->step, cap = B.cap;
     const int buf = (int)((step + 1) & 1);
-    const uint32_t sn = (uint32_t)(step + 1);
     const double* X = B.x[buf];
-    const double x = X[i], y = X[cap + i], z = X[2 * cap + i];
-    const unsigned long long id = B.id[buf][i];
-    double cx, cy, cz, bx, by, bz;
-    ion_terms<8>(P, B, buf, i, x, y, z, cx, cy, cz, bx, by, bz);
     double* T = B.pre;
-    T[i] = cx, T[cap + i] = cy, T[2 * cap + i] = cz;
-    T[3 * cap + i] = bx, T[4 * cap + i] = by, T[5 * cap + i] = bz;
-    const uint4 w = philox(P, id, sn, ST_COLL);
-    if ((unsigned long long)w.x >= P.Tcoll) return;
-    double vx, vy, vz;
-    collision_velocity(P, id, sn, vx, vy, vz);
-    B.coll_v[i] = vx;
-    B.coll_v[cap + i] = vy;
-    B.coll_v[2 * cap + i] = vz;
+    if (blockIdx.y == 2) {
+        const uint32_t sn = (uint32_t)(step + 1);
+        const unsigned long long id = B.id[buf][i];
+        const uint4 w = philox(P, id, sn, ST_COLL);
+        if ((unsigned long long)w.x >= P.Tcoll) return;
+        double vx, vy, vz;
+        collision_velocity(P, id, sn, vx, vy, vz);
+        B.coll_v[i] = vx;
+        B.coll_v[cap + i] = vy;
+        B.coll_v[2 * cap + i] = vz;
+        return;
+    }
+    const double x = X[i], y = X[cap + i], z = X[2 * cap + i];
+    double a, b, c;
+    if (blockIdx.y == 0) {
+        if (!P.cp_on) return;
+        close_pairs_of<8>(P, B, buf, i, x, y, z, a, b, c);
+    } else {
+        T += 3 * cap;
+        ion_field(P, x, y, z, a, b, c);
+    }
+    T[i] = a, T[cap + i] = b, T[2 * cap + i] = c;
 }
 
 int launch_ion_terms(const Phys& P, const Bufs& B, cudaStream_t s)
 {
     if (P.N == 0) return 0;
-    k_ion_terms<<<(P.N + KICK_BT - 1) / KICK_BT, KICK_BT, 0, s>>>(P, B);
+    k_ion_terms<<<dim3((P.N + TERMS_BT - 1) / TERMS_BT, 3), TERMS_BT, 0, s>>>(P, B);
     return (int)cudaGetLastError();
 }
 
@@ -209,12 +222,13 @@ int launch_grains(const Phys& P, const Bufs& B, cudaStream_t s)
     return (int)cudaGetLastError();
 }
 
-// Phi(z0) and phi(z0), z0 = -u / sig, after the tabulated inverse flux CDFs
+// Phi(z0), phi(z0) (z0 = -u / sig) and 1 / sig, after the tabulated inverse flux CDFs
 __global__ void k_vtab_consts(double* vtab, double u, double sig)
 {
     const double z0 = -u / sig;
     vtab[2 * (VTAB_K + 1)] = ncdf(z0);
     vtab[2 * (VTAB_K + 1) + 1] = npdf(z0);
+    vtab[2 * (VTAB_K + 1) + 2] = 1.0 / sig;
 }
 
 int launch_vtab_consts(double* vtab, double u, double sig, cudaStream_t s)
@@ -478,7 +492,8 @@ static int ck(cudaError_t e)
     return e == cudaSuccess ? 0 : (int)e;
 }
 
-int push_tile() { return PUSH_BT; }
+// 64-ion tiles up to one per SM: the scan's FP64 (two lanes per clock and SM) spreads out
+int push_tile(int N) { return N <= PUSH_SMALL_MAX ? PUSH_BT_SMALL : PUSH_BT; }
 int kick_block() { return KICK_BT; }
 
 int launch_init_ions(const Phys& P, const Bufs& B, cudaStream_t s)
@@ -510,8 +525,9 @@ int launch_push_scan(const Phys& P, const Bufs& B, cudaStream_t s)
 {
     if (P.N == 0) return 0;
     const double ls_inv = 1.4426950408889634 * P.lam_inv;
-    const int n_tiles = (P.N + PUSH_BT - 1) / PUSH_BT;
-    k_push_scan<PUSH_BT><<<n_tiles, PUSH_BT, 0, s>>>(P, B, n_tiles, ls_inv);
+    const int bt = push_tile(P.N), n_tiles = (P.N + bt - 1) / bt;
+    if (bt == PUSH_BT) k_push_scan<PUSH_BT><<<n_tiles, PUSH_BT, 0, s>>>(P, B, n_tiles, ls_inv);
+    else k_push_scan<PUSH_BT_SMALL><<<n_tiles, PUSH_BT_SMALL, 0, s>>>(P, B, n_tiles, ls_inv);
     return ck(cudaGetLastError());
 }
 
