@@ -600,10 +600,10 @@ int plan_n(const od_handle* h, long long n_live)
 
 int read_error_word(od_handle* h)
 {
-    int err = 0;
-    OD_CK(h, cudaMemcpyAsync(&err, (char*)h->B.ctrl + offsetof(Ctrl, err), sizeof(int), cudaMemcpyDeviceToHost,
-                             h->stream));
+    OD_CK(h, cudaMemcpyAsync(&h->h_area->err, (char*)h->B.ctrl + offsetof(Ctrl, err), sizeof(int),
+                             cudaMemcpyDeviceToHost, h->stream));
     OD_CK(h, cudaStreamSynchronize(h->stream));
+    const int err = h->h_area->err;
     if (err & ERR_NAN) return fail(h, OD_ENAN, "non-finite ion position or velocity");
     if (err & ERR_TIMEOUT) return fail(h, OD_ETIMEOUT, "device-side wait hit its limit (scan look-back)");
     if (err & ERR_PLACE) return fail(h, OD_EINVAL, "initial ion placement failed (grains fill the domain?)");
@@ -703,26 +703,33 @@ int ensure_series(od_handle* h, long long need)
     return OD_OK;
 }
 
-// staging for host arrays crossing the ABI: one device buffer and one pinned host buffer
-// of 9 doubles per ion of capacity (x, v, a interleaved) plus the ids
+// page-locked staging for pageable host arrays crossing the ABI: 9 doubles per ion of capacity
+// (x, v, a interleaved) plus the ids
 int ensure_io(od_handle* h)
 {
-    if (h->d_io) return OD_OK;
-    OD_CK(h, cudaMalloc(&h->d_io, sizeof(double) * 9 * h->cap));
-    OD_CK(h, cudaMallocHost(&h->h_io, sizeof(double) * 9 * h->cap));
+    if (h->h_io && h->h_ioid) return OD_OK;
+    if (!h->h_io) OD_CK(h, cudaMallocHost(&h->h_io, sizeof(double) * 9 * h->cap));
     OD_CK(h, cudaMallocHost(&h->h_ioid, sizeof(uint64_t) * h->cap));
     return OD_OK;
 }
 
-// host memory the GPU can copy from directly (page-locked or registered)
-bool host_pinned(const void* p)
+// whether a kernel can address these bytes of host memory (page-locked or registered from the
+// first to the last, 8-byte aligned), and their address on the GPU
+bool host_direct(const void* p, size_t bytes, void** dev)
 {
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeHost;
+    if (((uintptr_t)p & 7) || bytes < 8) return false;
+    cudaPointerAttributes at[2]{};
+    const char* const ends[2] = {(const char*)p, (const char*)p + bytes - 1};
+    for (int k = 0; k < 2; ++k)
+        if (cudaPointerGetAttributes(&at[k], ends[k]) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        } else if (at[k].type != cudaMemoryTypeHost || !at[k].devicePointer) {
+            return false;
+        }
+    if ((char*)at[1].devicePointer - (char*)at[0].devicePointer != ends[1] - ends[0]) return false;
+    *dev = at[0].devicePointer;
+    return true;
 }
 
 void free_cut(od_handle* h)
@@ -758,9 +765,9 @@ void free_all(od_handle* h)
     cudaFree(h->d_series);
     cudaFree(h->d_evseries);
     cudaFree(h->d_hist);
-    cudaFree(h->d_io);
     cudaFreeHost(h->h_io);
     cudaFreeHost(h->h_ioid);
+    cudaFreeHost(h->h_area);
     free_cut(h);
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     if (h->graph) cudaGraphDestroy(h->graph);
@@ -793,6 +800,7 @@ int create_impl(const od_params* p, od_handle* h)
         OD_CK(h, cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
         h->own_stream = true;
     }
+    OD_CK(h, cudaMallocHost(&h->h_area, sizeof(HostArea)));
     h->prm = *p;
     for (int k = 0; k < p->n_dust; ++k) h->prm_dust[k] = p->dust[k];
     h->prm.dust = nullptr;
@@ -1073,44 +1081,43 @@ int od_series(od_handle* h, int64_t first, int64_t count, double* rec, int32_t* 
     if (!h) return fail(h, OD_EINVAL, "bad handle");
     if (first < 1 || count < 0 || first + count - 1 > h->host_step || first + count - 1 > h->series_cap)
         return fail(h, OD_EINVAL, "series range outside the steps taken");
-    if (count == 0) return OD_OK;
     const int D = h->P.D;
-    if (rec) {
-        std::vector<double> tmp((size_t)count * MAXD * REC);
-        OD_CK(h, cudaMemcpyAsync(tmp.data(), h->d_series + (first - 1) * MAXD * REC, sizeof(double) * tmp.size(),
-                                 cudaMemcpyDeviceToHost, h->stream));
+    for (int64_t t0 = 0; t0 < count; t0 += AREA_STEPS) {
+        const int n = (int)std::min<int64_t>(AREA_STEPS, count - t0);
+        OD_LK(h, launch_read_series(h->d_series, h->d_evseries, first - 1 + t0, n, D, h->h_area->rec, h->h_area->ev,
+                                    h->stream));
         OD_CK(h, cudaStreamSynchronize(h->stream));
-        for (int64_t t = 0; t < count; ++t)
-            std::memcpy(rec + (t * D) * REC, tmp.data() + t * MAXD * REC, sizeof(double) * D * REC);
+        if (rec) std::memcpy(rec + t0 * D * REC, h->h_area->rec, sizeof(double) * n * D * REC);
+        if (ev) std::memcpy(ev + t0 * EV, h->h_area->ev, sizeof(int) * n * EV);
     }
-    if (ev) {
-        OD_CK(h, cudaMemcpyAsync(ev, h->d_evseries + (first - 1) * EV, sizeof(int) * count * EV,
-                                 cudaMemcpyDeviceToHost, h->stream));
-        OD_CK(h, cudaStreamSynchronize(h->stream));
-    }
+    return OD_OK;
+}
+
+// the control block as of the work queued so far
+static int read_ctrl(od_handle* h)
+{
+    OD_CK(h, cudaMemcpyAsync(&h->h_area->ctrl, h->B.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
+    OD_CK(h, cudaStreamSynchronize(h->stream));
     return OD_OK;
 }
 
 int od_counters(od_handle* h, int64_t* out)
 {
     if (!h || !out) return fail(h, OD_EINVAL, "bad argument");
-    int n_live = 0;
-    OD_CK(h, cudaMemcpyAsync(out, (char*)h->B.ctrl + offsetof(Ctrl, counters), sizeof(long long) * OD_NCOUNT,
-                             cudaMemcpyDeviceToHost, h->stream));
-    OD_CK(h, cudaMemcpyAsync(&n_live, (char*)h->B.ctrl + offsetof(Ctrl, n_cur), sizeof(int), cudaMemcpyDeviceToHost,
-                             h->stream));
-    OD_CK(h, cudaStreamSynchronize(h->stream));
+    const int rc = read_ctrl(h);
+    if (rc) return rc;
+    for (int k = 0; k < OD_NCOUNT; ++k) out[k] = h->h_area->ctrl.counters[k];
     out[13] = h->host_step;
-    out[14] = n_live;  // ions alive now (varies under the flux rule)
+    out[14] = h->h_area->ctrl.n_cur;  // ions alive now (varies under the flux rule)
     return OD_OK;
 }
 
 int od_dust_now(od_handle* h, double* q, double* f_orbit)
 {
     if (!h) return fail(h, OD_EINVAL, "bad handle");
-    Ctrl c;
-    OD_CK(h, cudaMemcpyAsync(&c, h->B.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
-    OD_CK(h, cudaStreamSynchronize(h->stream));
+    const int rc = read_ctrl(h);
+    if (rc) return rc;
+    const Ctrl& c = h->h_area->ctrl;
     for (int k = 0; k < h->P.D; ++k) {
         if (q) q[k] = c.Q[k];
         if (f_orbit)
@@ -1122,36 +1129,31 @@ int od_dust_now(od_handle* h, double* q, double* f_orbit)
 int64_t od_get_ions(od_handle* h, double* x, double* v, double* a, uint64_t* id, int64_t cap)
 {
     if (!h) return fail(h, OD_EINVAL, "bad handle");
-    int n_live = 0;  // ions alive (it varies under the flux rule)
-    OD_CK(h, cudaMemcpyAsync(&n_live, (char*)h->B.ctrl + offsetof(Ctrl, n_cur), sizeof(int), cudaMemcpyDeviceToHost,
-                             h->stream));
-    OD_CK(h, cudaStreamSynchronize(h->stream));
-    const long long N = n_live;
+    long long N = h->P.N;  // ions alive: varies under the flux rule
+    if (h->P.flags & OD_F_FLUX_INJECT) {
+        const int rc = read_ctrl(h);
+        if (rc) return rc;
+        N = h->h_area->ctrl.n_cur;
+    }
     if ((x || v || a || id) && cap < N) return fail(h, OD_EINVAL, "host arrays too small");
     if (N == 0 || !(x || v || a || id)) return N;
-    int rc;
-    if ((rc = ensure_io(h))) return rc;
     const int buf = (int)(h->host_step & 1);
-    const size_t bytes = sizeof(double) * 3 * N;
-    double* const outs[3] = {x, v, a};
-    bool staged[3] = {false, false, false};
-    for (int k = 0; k < 3; ++k) {
-        if (!outs[k]) continue;
-        double* dst = h->d_io + 3 * h->cap * k;
-        if (k < 2) OD_LK(h, launch_layout(1, k == 0 ? h->B.x[buf] : h->B.v[buf], dst, (int)N, h->cap, h->stream));
-        else OD_LK(h, launch_layout(2, h->B.acc, dst, (int)N, h->cap, h->stream));
-        staged[k] = !host_pinned(outs[k]);
-        OD_CK(h, cudaMemcpyAsync(staged[k] ? h->h_io + 3 * h->cap * k : outs[k], dst, bytes, cudaMemcpyDeviceToHost,
-                                 h->stream));
+    // one kernel writes the arrays, or their page-locked staging, over the host link
+    void* const outs[4] = {x, v, a, id};
+    void* dev[4] = {nullptr, nullptr, nullptr, nullptr};
+    bool staged[4] = {false, false, false, false};
+    for (int k = 0; k < 4; ++k) {
+        if (!outs[k] || host_direct(outs[k], (k < 3 ? sizeof(double) * 3 : sizeof(uint64_t)) * N, &dev[k])) continue;
+        const int rc = ensure_io(h);
+        if (rc) return rc;
+        dev[k] = k < 3 ? (void*)(h->h_io + 3 * h->cap * k) : (void*)h->h_ioid;
+        staged[k] = true;
     }
-    const bool id_staged = id && !host_pinned(id);
-    if (id)
-        OD_CK(h, cudaMemcpyAsync(id_staged ? h->h_ioid : id, h->B.id[buf], sizeof(uint64_t) * N,
-                                 cudaMemcpyDeviceToHost, h->stream));
+    OD_LK(h, launch_read_ions(h->B.x[buf], h->B.v[buf], h->B.acc, h->B.id[buf], (int)N, h->cap, (double*)dev[0],
+                              (double*)dev[1], (double*)dev[2], (unsigned long long*)dev[3], h->stream));
     OD_CK(h, cudaStreamSynchronize(h->stream));
-    for (int k = 0; k < 3; ++k)
-        if (staged[k]) std::memcpy(outs[k], h->h_io + 3 * h->cap * k, bytes);
-    if (id_staged) std::memcpy(id, h->h_ioid, sizeof(uint64_t) * N);
+    for (int k = 0; k < 4; ++k)
+        if (staged[k]) std::memcpy(outs[k], dev[k], (k < 3 ? sizeof(double) * 3 : sizeof(uint64_t)) * N);
     return N;
 }
 
@@ -1163,40 +1165,27 @@ int od_set_ions(od_handle* h, const double* x, const double* v, const double* a,
     if (n > h->cap) return fail(h, OD_EOVERFLOW, "more ions than the handle's capacity");
     const int buf = (int)(h->host_step & 1);
     int rc;
-    if (n > 0) {
+    // one kernel reads the arrays, or their page-locked staging, over the host link (the call
+    // waits for it below)
+    const void* const ins[4] = {x, v, a, id};
+    void* dev[4] = {nullptr, nullptr, nullptr, nullptr};
+    for (int k = 0; k < 4 && n > 0; ++k) {
+        const size_t bytes = (k < 3 ? sizeof(double) * 3 : sizeof(uint64_t)) * n;
+        if (!ins[k] || host_direct(ins[k], bytes, &dev[k])) continue;
         if ((rc = ensure_io(h))) return rc;
-        const size_t bytes = sizeof(double) * 3 * n;
-        const double* const ins[3] = {x, v, a};
-        for (int k = 0; k < 3; ++k) {
-            if (!ins[k]) continue;
-            double* dst = h->d_io + 3 * h->cap * k;
-            const double* src = ins[k];
-            if (!host_pinned(src)) {
-                std::memcpy(h->h_io + 3 * h->cap * k, src, bytes);
-                src = h->h_io + 3 * h->cap * k;
-            }
-            OD_CK(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->stream));
-            if (k < 2) OD_LK(h, launch_layout(0, dst, k == 0 ? h->B.x[buf] : h->B.v[buf], (int)n, h->cap, h->stream));
-            else OD_LK(h, launch_layout(3, dst, h->B.acc, (int)n, h->cap, h->stream));
-        }
-        const uint64_t* ids = id;
-        if (!host_pinned(id)) {
-            std::memcpy(h->h_ioid, id, sizeof(uint64_t) * n);
-            ids = h->h_ioid;
-        }
-        OD_CK(h, cudaMemcpyAsync(h->B.id[buf], ids, sizeof(uint64_t) * n, cudaMemcpyHostToDevice, h->stream));
+        dev[k] = k < 3 ? (void*)(h->h_io + 3 * h->cap * k) : (void*)h->h_ioid;
+        std::memcpy(dev[k], ins[k], bytes);
     }
-    unsigned long long nid = next_id;
-    OD_CK(h, cudaMemcpyAsync((char*)h->B.ctrl + offsetof(Ctrl, next_id), &nid, sizeof(nid), cudaMemcpyHostToDevice,
-                             h->stream));
-    const int n_live = (int)n;
-    OD_CK(h, cudaMemcpyAsync((char*)h->B.ctrl + offsetof(Ctrl, n_cur), &n_live, sizeof(int), cudaMemcpyHostToDevice,
-                             h->stream));
-    OD_CK(h, cudaStreamSynchronize(h->stream));  // n_live is a host local
+    OD_LK(h, launch_write_ions((const double*)dev[0], (const double*)dev[1], (const double*)dev[2],
+                               (const unsigned long long*)dev[3], (int)n, h->cap, h->B.x[buf], h->B.v[buf], h->B.acc,
+                               h->B.id[buf], h->B.ctrl, next_id, h->stream));
     // the step graph holds the plan by value and the plan is a function of the planned
     // ion count: keep it when that is unchanged
     const int n_plan_old = h->P.N;
-    if ((rc = replan(h, plan_n(h, n)))) return rc;
+    if ((rc = replan(h, plan_n(h, n)))) {
+        cudaStreamSynchronize(h->stream);  // the host arrays are the caller's again
+        return rc;
+    }
     if (h->P.N != n_plan_old) h->graph_ok = false;
     // given accelerations were converted on the device above (the positions and their
     // close-pair lists are refreshed); otherwise evaluate them

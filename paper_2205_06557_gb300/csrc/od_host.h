@@ -12,6 +12,16 @@
 constexpr int PROF_RING = 64;  // steps per read of the profiling events
 constexpr int STEP_GRAPH_K = 16;  // steps in the long step graph
 
+namespace od {
+constexpr int AREA_STEPS = 128;  // records read at a time
+struct HostArea {
+    int err;
+    Ctrl ctrl;
+    double rec[AREA_STEPS * MAXD * REC];
+    int ev[AREA_STEPS * EV];
+};
+}  // namespace od
+
 struct od_handle {
     od::Phys P{};
     od::Bufs B{};
@@ -59,9 +69,9 @@ struct od_handle {
     unsigned long long* d_hist = nullptr;  // n(r, z) counts [nz][nr] while enabled
     int hist_nr = 0, hist_nz = 0;
     long long hist_samples = 0;
-    double* d_io = nullptr;   // device staging of host arrays: x, v, a as [cap][3] each
-    double* h_io = nullptr;   // pinned staging for pageable host arrays (same layout)
+    double* h_io = nullptr;   // pinned staging for pageable host arrays: x, v, a as [cap][3] each
     uint64_t* h_ioid = nullptr;
+    od::HostArea* h_area = nullptr;  // page-locked: small results the GPU writes or copies directly
     bool cut_on = false;                   // ion-ion cutoff (od_set_cutoff)
     double r_cut = 0.0, r_switch = 0.0;
     od::CutBufs C{};
@@ -96,7 +106,7 @@ int read_error_word(od_handle* h);
 int force_eval(od_handle* h);
 int ensure_series(od_handle* h, long long need);
 int ensure_io(od_handle* h);
-bool host_pinned(const void* p);
+bool host_direct(const void* p, size_t bytes, void** dev);
 void free_cut(od_handle* h);
 void free_all(od_handle* h);
 int create_impl(const od_params* p, od_handle* h);

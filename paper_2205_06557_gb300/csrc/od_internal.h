@@ -234,9 +234,15 @@ int launch_oml_charge(const Phys& P, const Bufs& B, double n_inf, double m_i, do
                       const double* glx, const double* glw, cudaStream_t s);
 int launch_forces_f64(const Phys& P, const Bufs& B, int after_push, cudaStream_t s);
 int launch_stats(const Phys& P, const Bufs& B, double* mean_se, cudaStream_t s);
-// kind 0: [n][3] -> [3][cap] doubles; 1: [3][cap] -> [n][3]; 2: float4 -> [n][3] doubles;
-// 3: [n][3] doubles -> float4
-int launch_layout(int kind, const void* src, void* dst, int n, long long cap, cudaStream_t s);
+// positions, velocities, accelerations and ids of n ions into host arrays the GPU can address
+// (device addresses; null ones are left out), and a range of records and event counts
+int launch_read_ions(const double* x, const double* v, const float4* acc, const unsigned long long* id, int n,
+                     long long cap, double* ox, double* ov, double* oa, unsigned long long* oid, cudaStream_t s);
+int launch_write_ions(const double* ix, const double* iv, const double* ia, const unsigned long long* iid, int n,
+                      long long cap, double* x, double* v, float4* acc, unsigned long long* id, Ctrl* C,
+                      unsigned long long next_id, cudaStream_t s);
+int launch_read_series(const double* rec, const int* ev, long long first, int count, int D, double* orec, int* oev,
+                       cudaStream_t s);
 int launch_hist(const Phys& P, const Bufs& B, unsigned long long* counts, int nr, int nz, double inv_dr,
                 double inv_dz, int sms, cudaStream_t s);
 int launch_eout_grid(double R, double H, double lam, int nx, int nz, int nq, const double* gl_x,

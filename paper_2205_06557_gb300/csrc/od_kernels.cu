@@ -670,55 +670,120 @@ int launch_kick_step(const Phys& P, const Bufs& B, const ForceArgs& F, cudaStrea
     return ck(cudaGetLastError());
 }
 
-// host interface layouts: the ABI's interleaved [n][3] arrays <-> the device's [3][cap]
-// structure of arrays (and the float4 accelerations), converted on the device so that a
-// host array moves as one contiguous copy
-__global__ void k_aos_to_soa(const double* __restrict__ aos, double* __restrict__ soa, int n, long long cap)
+// The ABI's interleaved [n][3] host arrays <-> the device's [3][cap] structure of arrays (and the
+// float4 accelerations), straight over the host link (the arrays, or their staging, are
+// page-locked): one launch instead of a layout kernel and a copy per array.  Each block turns
+// 128 ions' values round in shared memory, so that host memory is touched in whole
+// consecutive words.  Reading 2,000 ions back 60 -> 27 us, 1,000,000 ions 522 -> 442 us.
+constexpr int READ_BT = 128;
+
+__device__ __forceinline__ void read_rows(const double* soa, long long cap, double* out, int i0, int n, double* s)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    soa[i] = aos[3 * (long long)i];
-    soa[cap + i] = aos[3 * (long long)i + 1];
-    soa[2 * cap + i] = aos[3 * (long long)i + 2];
+    const int i = i0 + threadIdx.x;
+    __syncthreads();
+    if (i < n)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) s[3 * threadIdx.x + d] = soa[d * cap + i];
+    __syncthreads();
+    const int m = 3 * min(READ_BT, n - i0);
+    for (int e = threadIdx.x; e < m; e += READ_BT) out[3 * (long long)i0 + e] = s[e];
 }
 
-__global__ void k_soa_to_aos(const double* __restrict__ soa, double* __restrict__ aos, int n, long long cap)
+__global__ void __launch_bounds__(READ_BT)
+    k_read_ions(const double* x, const double* v, const float4* acc, const unsigned long long* id, int n, long long cap,
+                double* ox, double* ov, double* oa, unsigned long long* oid)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    aos[3 * (long long)i] = soa[i];
-    aos[3 * (long long)i + 1] = soa[cap + i];
-    aos[3 * (long long)i + 2] = soa[2 * cap + i];
+    __shared__ double s[3 * READ_BT];
+    const int i0 = blockIdx.x * READ_BT, i = i0 + threadIdx.x;
+    if (ox) read_rows(x, cap, ox, i0, n, s);
+    if (ov) read_rows(v, cap, ov, i0, n, s);
+    if (oa) {
+        __syncthreads();
+        if (i < n) {
+            const float4 a = acc[i];
+            s[3 * threadIdx.x] = a.x, s[3 * threadIdx.x + 1] = a.y, s[3 * threadIdx.x + 2] = a.z;
+        }
+        __syncthreads();
+        const int m = 3 * min(READ_BT, n - i0);
+        for (int e = threadIdx.x; e < m; e += READ_BT) oa[3 * (long long)i0 + e] = s[e];
+    }
+    if (oid && i < n) oid[i] = id[i];
 }
 
-__global__ void k_acc_to_aos(const float4* __restrict__ acc, double* __restrict__ aos, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float4 a = acc[i];
-    aos[3 * (long long)i] = a.x;
-    aos[3 * (long long)i + 1] = a.y;
-    aos[3 * (long long)i + 2] = a.z;
-}
-
-__global__ void k_aos_to_acc(const double* __restrict__ aos, float4* __restrict__ acc, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    acc[i] = make_float4((float)aos[3 * (long long)i], (float)aos[3 * (long long)i + 1], (float)aos[3 * (long long)i + 2],
-                         0.f);
-}
-
-int launch_layout(int kind, const void* src, void* dst, int n, long long cap, cudaStream_t s)
+int launch_read_ions(const double* x, const double* v, const float4* acc, const unsigned long long* id, int n,
+                     long long cap, double* ox, double* ov, double* oa, unsigned long long* oid, cudaStream_t s)
 {
     if (n <= 0) return 0;
-    const int g = (n + 255) / 256;
-    switch (kind) {
-    case 0: k_aos_to_soa<<<g, 256, 0, s>>>((const double*)src, (double*)dst, n, cap); break;
-    case 1: k_soa_to_aos<<<g, 256, 0, s>>>((const double*)src, (double*)dst, n, cap); break;
-    case 2: k_acc_to_aos<<<g, 256, 0, s>>>((const float4*)src, (double*)dst, n); break;
-    default: k_aos_to_acc<<<g, 256, 0, s>>>((const double*)src, (float4*)dst, n); break;
+    k_read_ions<<<(n + READ_BT - 1) / READ_BT, READ_BT, 0, s>>>(x, v, acc, id, n, cap, ox, ov, oa, oid);
+    return ck(cudaGetLastError());
+}
+
+// and the other way: a replaced state from host arrays the GPU can address (a may be null), with
+// the control block's count and next id
+__device__ __forceinline__ void write_rows(const double* in, double* soa, long long cap, int i0, int n, double* s)
+{
+    const int i = i0 + threadIdx.x, m = 3 * min(READ_BT, n - i0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < m; e += READ_BT) s[e] = in[3 * (long long)i0 + e];
+    __syncthreads();
+    if (i < n)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) soa[d * cap + i] = s[3 * threadIdx.x + d];
+}
+
+__global__ void __launch_bounds__(READ_BT)
+    k_write_ions(const double* ix, const double* iv, const double* ia, const unsigned long long* iid, int n,
+                 long long cap, double* x, double* v, float4* acc, unsigned long long* id, Ctrl* C,
+                 unsigned long long next_id)
+{
+    __shared__ double s[3 * READ_BT];
+    const int i0 = blockIdx.x * READ_BT, i = i0 + threadIdx.x;
+    if (i0 < n) {
+        write_rows(ix, x, cap, i0, n, s);
+        write_rows(iv, v, cap, i0, n, s);
+        if (ia) {
+            const int m = 3 * min(READ_BT, n - i0);
+            __syncthreads();
+            for (int e = threadIdx.x; e < m; e += READ_BT) s[e] = ia[3 * (long long)i0 + e];
+            __syncthreads();
+            if (i < n)
+                acc[i] = make_float4((float)s[3 * threadIdx.x], (float)s[3 * threadIdx.x + 1],
+                                     (float)s[3 * threadIdx.x + 2], 0.f);
+        }
+        if (i < n) id[i] = iid[i];
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        C->next_id = next_id;
+        C->n_cur = n;
+    }
+}
+
+int launch_write_ions(const double* ix, const double* iv, const double* ia, const unsigned long long* iid, int n,
+                      long long cap, double* x, double* v, float4* acc, unsigned long long* id, Ctrl* C,
+                      unsigned long long next_id, cudaStream_t s)
+{
+    k_write_ions<<<std::max(1, (n + READ_BT - 1) / READ_BT), READ_BT, 0, s>>>(ix, iv, ia, iid, n, cap, x, v, acc, id, C,
+                                                                            next_id);
+    return ck(cudaGetLastError());
+}
+
+// reads of a range of records and event counts (the D grains' records only)
+__global__ void k_read_series(const double* rec, const int* ev, long long first, int count, int D, double* orec, int* oev)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nr = count * D * REC;
+    if (i < nr) {
+        const int t = i / (D * REC), e = i % (D * REC);
+        orec[i] = rec[(first + t) * MAXD * REC + e];
+    }
+    if (i < count * EV) oev[i] = ev[first * EV + i];
+}
+
+int launch_read_series(const double* rec, const int* ev, long long first, int count, int D, double* orec, int* oev,
+                       cudaStream_t s)
+{
+    const int m = count * std::max(D * REC, EV);
+    k_read_series<<<(m + 255) / 256, 256, 0, s>>>(rec, ev, first, count, D, orec, oev);
     return ck(cudaGetLastError());
 }
 
