@@ -619,7 +619,7 @@ int force_eval(od_handle* h)
 {
     OD_LK(h, launch_fpos(h->P, h->B, (int)(h->host_step & 1), h->stream));
     OD_LK(h, launch_pairs(h, 0));
-    OD_LK(h, launch_kick(h->P, h->B, h->F, 1, h->stream));  // with the grain tail
+    OD_LK(h, launch_kick(h->P, h->B, h->F, h->stream));  // with the grain tail
     return OD_OK;
 }
 
@@ -868,12 +868,12 @@ int create_impl(const od_params* p, od_handle* h)
     OD_CK(h, cudaMalloc(&B.inj, sizeof(Inj) * h->cap));
     OD_CK(h, cudaMalloc(&B.rem, sizeof(Rem) * h->cap));
     OD_CK(h, cudaMalloc(&B.inj_ahead, sizeof(Inj) * INJ_AHEAD));
+    OD_CK(h, cudaMalloc(&B.coll_v, sizeof(double) * 3 * h->cap));
+    OD_CK(h, cudaMalloc(&B.pre, sizeof(double) * 6 * h->cap));
+    OD_CK(h, cudaMalloc(&B.felt, sizeof(Felt)));
+    OD_CK(h, cudaMemsetAsync(B.felt, 0, sizeof(Felt), h->stream));
     if (!h->batch_member) {
         // single runs compute what does not need the pair forces beside them, on more streams
-        OD_CK(h, cudaMalloc(&B.coll_v, sizeof(double) * 3 * h->cap));
-        OD_CK(h, cudaMalloc(&B.pre, sizeof(double) * 6 * h->cap));
-        OD_CK(h, cudaMalloc(&B.felt, sizeof(Felt)));
-        OD_CK(h, cudaMemsetAsync(B.felt, 0, sizeof(Felt), h->stream));
         OD_CK(h, cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
         for (int k = 0; k < 3; ++k) {
             OD_CK(h, cudaStreamCreateWithFlags(&h->aux[k], cudaStreamNonBlocking));

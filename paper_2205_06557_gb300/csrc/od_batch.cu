@@ -1,16 +1,20 @@
 // Batched persistent step: many independent runs of uneven ion count advance one
 // step in ONE kernel launch (replayed from a CUDA graph).
 //
-// Every run's step is split into tasks of its four phases (scan tiles of 128 ions,
-// pair units of one target tile x one source chunk, kick tiles, one grain-tail task).
+// Every run's step is split into tasks (BatchTask): scan tiles of 128 ions; pair units of one
+// target tile x one source chunk (or tile pairs); side tiles of 128 ions (the ion terms and
+// the grain sums, which need the positions but not the pair forces); a grain tail; kick tiles.
 // A persistent grid of at most the resident number of CTAs takes tasks from a global
-// counter in phase-major order (all scan tiles, then all pair units, then all kick
-// tiles, then all grain tails; runs in order inside each phase).  A task of phase p of
-// run r first waits until run r's phase p-1 counter reaches its target; every task it
-// waits for was handed out earlier to a CTA that is running, so the waits end (and
+// counter, all scan tiles first, then all pair units, side tiles, tails and kick tiles (runs
+// in order inside each kind), so the side tiles and tails fill the CTAs that run out of pair
+// units while others still work on theirs.  A task first waits until the counters of the
+// kinds it depends on (of its run) reach their targets: pair units and side tiles for the
+// scan, the tail for the side tiles, the kick for the pair units and the side tiles; every
+// task waited for was handed out earlier to a CTA that is running, so the waits end (and
 // each is bounded anyway: it gives up after spin_limit polls and sets an error).
-// The counters only grow (target = (batch step + 1) x tasks per phase), so nothing
+// The counters only grow (target = (batch step + 1) x tasks of the kind), so nothing
 // is reset between launches; the last CTA to leave advances the batch step.
+// 48 runs of 2,171 ions (ordered units): @BATCH@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -30,20 +34,73 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64c(const unsigned lon
     return v;
 }
 
-// phase_end: cumulative task-index ends of phases 0..3.  tune = 1: a tuning launch whose
-// task list holds only pair units and kick tiles; the pair units do not wait, the kick
-// tiles wait for their run's pair units as in a step (on the tuning launch's own counters)
-// and evaluate accelerations only (kick mode 1: no velocity update, no collisions), so the
-// runs' states are not changed.
+// The ion terms and the grain side of one tile (kick_body<..., true> and dust_body follow): what
+// k_ion_terms and k_grains do for a single run.
+template <int BT>
+__device__ __forceinline__ void side_tile(const Phys& P, const Bufs& B, int tile)
+{
+    Ctrl* C = B.ctrl;
+    const int i = tile * BT + threadIdx.x;
+    const bool live = i < C->n_cur;
+    const long long step = B.felt->step, cap = B.cap;
+    const int buf = (int)((step + 1) & 1);
+    const uint32_t sn = (uint32_t)(step + 1);
+    double x = 0, y = 0, z = 0;
+    int coll = 0;
+    if (live) {
+        const double* X = B.x[buf];
+        x = X[i], y = X[cap + i], z = X[2 * cap + i];
+        const unsigned long long id = B.id[buf][i];
+        double* T = B.pre;
+        double a, b, c;
+        if (P.cp_on) {
+            close_pairs_of<1>(P, B, buf, i, x, y, z, a, b, c);
+            T[i] = a, T[cap + i] = b, T[2 * cap + i] = c;
+        }
+        ion_field(P, x, y, z, a, b, c);
+        T[3 * cap + i] = a, T[4 * cap + i] = b, T[5 * cap + i] = c;
+        const uint4 w = philox(P, id, sn, ST_COLL);
+        if ((unsigned long long)w.x < P.Tcoll) {
+            collision_velocity(P, id, sn, a, b, c);
+            B.coll_v[i] = a, B.coll_v[cap + i] = b, B.coll_v[2 * cap + i] = c;
+            coll = 1;
+        }
+    }
+    const unsigned bc = __ballot_sync(0xffffffffu, coll);
+    if ((threadIdx.x & 31) == 0 && bc) atomicAdd(&C->ev_step[12], __popc(bc));
+    grain_sums<BT>(P, B, live, x, y, z, tile);
+}
+
+// bounded wait of the whole CTA for a run's counter to reach target
+__device__ __forceinline__ void wait_count(const unsigned long long* cnt, unsigned long long target, long long spin_limit,
+                                           BatchCtrl* bc)
+{
+    if (threadIdx.x == 0) {
+        long long spins = 0;
+        unsigned ns = 64;
+        while (ld_acquire_u64c(cnt) < target) {
+            if (++spins > spin_limit) {
+                atomicOr(&bc->err, ERR_TIMEOUT);
+                break;
+            }
+            __nanosleep(ns);
+            if (ns < 2048) ns *= 2;
+        }
+    }
+    __syncthreads();
+}
+
+// A task is (kind << 28 | run, index within the kind).  Tuning launches hold only pair units
+// and BT_FORCES kick tiles (accelerations only: no velocity update, no collisions) on counters of their own; their pair units do not wait, so the runs' states are
+// not changed.
 // held to 128 registers: four CTAs of 128 per SM
 template <int IPT>
 __global__ void __launch_bounds__(BATCH_BT, 65536 / (BATCH_BT * 128))
-    k_batch_step(const RunDesc* __restrict__ runs, const int2* __restrict__ tasks, int4 phase_end, long long T,
-                 BatchCtrl* bc, unsigned long long* done, int R, long long spin_limit, int tune)
+    k_batch_step(const RunDesc* __restrict__ runs, const int2* __restrict__ tasks, long long T, BatchCtrl* bc,
+                 unsigned long long* done, int R, long long spin_limit, int tune)
 {
     __shared__ SymShared<BATCH_BT / 32, BATCH_BT * IPT> sym;
     __shared__ long long s_task;
-    __shared__ int s_timeout;
     const unsigned long long bstep = bc->step;
     // every launch draws exactly T + gridDim.x tickets (T tasks plus one failing draw per CTA)
     const unsigned long long base = bstep * (unsigned long long)(T + gridDim.x);
@@ -54,34 +111,14 @@ __global__ void __launch_bounds__(BATCH_BT, 65536 / (BATCH_BT * 128))
         const long long t = s_task;
         if (t >= T) break;
         const int2 tk = tasks[t];
-        const RunDesc& d = runs[tk.x];
-        const int phase = t < phase_end.x ? 0 : t < phase_end.y ? 1 : t < phase_end.z ? 2 : 3;
-        if (phase > 1 || (phase == 1 && !tune)) {
-            // wait for the previous phase of this run
-            if (threadIdx.x == 0) {
-                const unsigned long long per = phase == 1 ? (unsigned long long)d.nA
-                                                          : phase == 2 ? (unsigned long long)d.F.U
-                                                                       : (unsigned long long)d.nK;
-                const unsigned long long target = (bstep + 1) * per;
-                const unsigned long long* cnt = done + (long long)(phase - 1) * R + tk.x;
-                long long spins = 0;
-                unsigned ns = 64;
-                s_timeout = 0;
-                while (ld_acquire_u64c(cnt) < target) {
-                    if (++spins > spin_limit) {
-                        s_timeout = 1;
-                        atomicOr(&bc->err, ERR_TIMEOUT);
-                        break;
-                    }
-                    __nanosleep(ns);
-                    if (ns < 2048) ns *= 2;
-                }
-            }
-            __syncthreads();
-        }
-        switch (phase) {
-        case 0: push_scan_body<BATCH_BT>(d.P, d.B, d.nA, 1.4426950408889634 * d.P.lam_inv, tk.y); break;
-        case 1:
+        const int kind = (unsigned)tk.x >> 28, r = tk.x & ((1 << 28) - 1);
+        const RunDesc& d = runs[r];
+        unsigned long long* cnt = done + r;  // [0] scan tiles, [R] pair units, [2 R] side tiles
+        const unsigned long long turn = bstep + 1;
+        switch (kind) {
+        case BT_SCAN: push_scan_body<BATCH_BT>(d.P, d.B, d.nA, 1.4426950408889634 * d.P.lam_inv, tk.y); break;
+        case BT_PAIR:
+            if (!tune) wait_count(cnt, turn * d.nA, spin_limit, bc);
             if (d.F.sym) {
                 int I, J;
                 tri_unit(tk.y, d.F.JS, I, J);
@@ -90,13 +127,29 @@ __global__ void __launch_bounds__(BATCH_BT, 65536 / (BATCH_BT * 128))
                 forces_unit<BATCH_BT, IPT>(d.B.fpos, d.B.part, d.F, tk.y / d.F.JS, tk.y % d.F.JS, sym.sj);
             }
             break;
-        case 2: kick_body<BATCH_BT, 1>(d.P, d.B, d.F, tune ? 1 : 0, tk.y); break;
-        default: dust_body<false>(d.P, d.B, d.nK, 0); break;
+        case BT_SIDE:
+            wait_count(cnt, turn * d.nA, spin_limit, bc);
+            side_tile<BATCH_BT>(d.P, d.B, tk.y);
+            break;
+        case BT_TAIL:
+            wait_count(cnt + 2 * R, turn * d.nK, spin_limit, bc);
+            dust_body<false>(d.P, d.B, d.nK, 0);
+            break;
+        case BT_KICK:
+            wait_count(cnt + R, turn * (unsigned long long)d.F.U, spin_limit, bc);
+            wait_count(cnt + 2 * R, turn * d.nK, spin_limit, bc);
+            kick_body<BATCH_BT, 1, true>(d.P, d.B, d.F, tk.y);
+            break;
+        default:
+            wait_count(cnt + R, turn * (unsigned long long)d.F.U, spin_limit, bc);
+            kick_body<BATCH_BT, 1>(d.P, d.B, d.F, tk.y);
+            break;
         }
-        // publish completion of this task to the run's phase counter
+        if (kind > BT_SIDE) continue;  // nothing in this launch waits for it
+        // publish completion of this task to the run's counter of its kind
         __threadfence();
         __syncthreads();
-        if (threadIdx.x == 0 && phase < 3) atomicAdd(done + (long long)phase * R + tk.x, 1ull);
+        if (threadIdx.x == 0) atomicAdd(cnt + (long long)kind * R, 1ull);
     }
     if (threadIdx.x == 0) {
         __threadfence();
@@ -123,18 +176,18 @@ int batch_blocks_per_sm(int ipt)
     return nb > 0 ? nb : 1;
 }
 
-int launch_batch(int ipt, int grid, const RunDesc* runs, const int2* tasks, int4 phase_end, long long T,
-                 BatchCtrl* bc, unsigned long long* done, int R, long long spin_limit, int tune, cudaStream_t s)
+int launch_batch(int ipt, int grid, const RunDesc* runs, const int2* tasks, long long T, BatchCtrl* bc,
+                 unsigned long long* done, int R, long long spin_limit, int tune, cudaStream_t s)
 {
     switch (ipt) {
     case 2:
-        k_batch_step<2><<<grid, BATCH_BT, 0, s>>>(runs, tasks, phase_end, T, bc, done, R, spin_limit, tune);
+        k_batch_step<2><<<grid, BATCH_BT, 0, s>>>(runs, tasks, T, bc, done, R, spin_limit, tune);
         break;
     case 4:
-        k_batch_step<4><<<grid, BATCH_BT, 0, s>>>(runs, tasks, phase_end, T, bc, done, R, spin_limit, tune);
+        k_batch_step<4><<<grid, BATCH_BT, 0, s>>>(runs, tasks, T, bc, done, R, spin_limit, tune);
         break;
     default:
-        k_batch_step<8><<<grid, BATCH_BT, 0, s>>>(runs, tasks, phase_end, T, bc, done, R, spin_limit, tune);
+        k_batch_step<8><<<grid, BATCH_BT, 0, s>>>(runs, tasks, T, bc, done, R, spin_limit, tune);
         break;
     }
     const cudaError_t e = cudaGetLastError();

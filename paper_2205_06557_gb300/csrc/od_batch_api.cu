@@ -20,13 +20,12 @@ struct od_batch {
     bool own_stream = false;
     RunDesc* d_runs = nullptr;
     int2* d_tasks = nullptr;
-    int2* d_tasks_f = nullptr;          // tuning: pair units, then kick tiles
-    unsigned long long* d_done = nullptr;
-    unsigned long long* d_done_f = nullptr;  // phase counters of the tuning launches
+    int2* d_tasks_f = nullptr;          // tuning: pair units, then accelerations
+    unsigned long long* d_done = nullptr;    // tasks done per run: scan tiles [R], pair units [R], side tiles [R]
+    unsigned long long* d_done_f = nullptr;  // those of the tuning launches
     BatchCtrl* d_bc = nullptr;
     BatchCtrl* d_bc_f = nullptr;
     long long T = 0, T_f = 0;
-    int4 phase_end{0, 0, 0, 0}, phase_end_f{0, 0, 0, 0};
     int ipt = 2, jc = 4096, grid = 1, sms = 1;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -60,7 +59,10 @@ int batch_build(od_batch* b)
 {
     const int R = (int)b->runs.size();
     std::vector<RunDesc> desc(R);
-    std::vector<int2> tA, tF, tK, tD;
+    std::vector<int2> all[BT_FORCES + 1];  // tasks by kind
+    auto add = [&](int kind, int r, long long n) {
+        for (long long i = 0; i < n; ++i) all[kind].push_back(make_int2(kind << 28 | r, (int)i));
+    };
     for (int r = 0; r < R; ++r) {
         od_handle* h = b->runs[r];
         h->F = batch_plan(h->P.N, b->ipt, b->jc);
@@ -78,22 +80,17 @@ int batch_build(od_batch* b)
         desc[r].nK = desc[r].nA;
         if (desc[r].nA > h->scan_tiles_cap || desc[r].nK > h->nb_cap)
             return bfail(b, OD_EINVAL, "batch: run " + std::to_string(r) + " has more scan or kick tiles than its buffers");
-        for (int i = 0; i < desc[r].nA; ++i) tA.push_back(make_int2(r, i));
-        for (long long u = 0; u < h->F.U; ++u) tF.push_back(make_int2(r, (int)u));
-        for (int i = 0; i < desc[r].nK; ++i) tK.push_back(make_int2(r, i));
-        tD.push_back(make_int2(r, 0));
+        add(BT_SCAN, r, desc[r].nA);
+        add(BT_PAIR, r, h->F.U);
+        add(BT_SIDE, r, desc[r].nK);
+        add(BT_TAIL, r, 1);
+        add(BT_KICK, r, desc[r].nK);
+        add(BT_FORCES, r, desc[r].nK);
     }
-    std::vector<int2> all;
-    all.insert(all.end(), tA.begin(), tA.end());
-    all.insert(all.end(), tF.begin(), tF.end());
-    all.insert(all.end(), tK.begin(), tK.end());
-    all.insert(all.end(), tD.begin(), tD.end());
-    b->phase_end = make_int4((int)tA.size(), (int)(tA.size() + tF.size()), (int)(tA.size() + tF.size() + tK.size()),
-                             (int)all.size());
-    b->T = (long long)all.size();
-    std::vector<int2> fk(tF);
-    fk.insert(fk.end(), tK.begin(), tK.end());
-    b->phase_end_f = make_int4(0, (int)tF.size(), (int)fk.size(), (int)fk.size());
+    std::vector<int2> step, fk(all[BT_PAIR]);
+    for (int k = BT_SCAN; k <= BT_KICK; ++k) step.insert(step.end(), all[k].begin(), all[k].end());
+    fk.insert(fk.end(), all[BT_FORCES].begin(), all[BT_FORCES].end());
+    b->T = (long long)step.size();
     b->T_f = (long long)fk.size();
     cudaFree(b->d_runs);
     cudaFree(b->d_tasks);
@@ -101,10 +98,10 @@ int batch_build(od_batch* b)
     b->d_runs = nullptr;
     b->d_tasks = b->d_tasks_f = nullptr;
     OD_BCK(b, cudaMalloc(&b->d_runs, sizeof(RunDesc) * R));
-    OD_BCK(b, cudaMalloc(&b->d_tasks, sizeof(int2) * std::max<size_t>(all.size(), 1)));
+    OD_BCK(b, cudaMalloc(&b->d_tasks, sizeof(int2) * std::max<size_t>(step.size(), 1)));
     OD_BCK(b, cudaMalloc(&b->d_tasks_f, sizeof(int2) * std::max<size_t>(fk.size(), 1)));
     OD_BCK(b, cudaMemcpyAsync(b->d_runs, desc.data(), sizeof(RunDesc) * R, cudaMemcpyHostToDevice, b->stream));
-    OD_BCK(b, cudaMemcpyAsync(b->d_tasks, all.data(), sizeof(int2) * all.size(), cudaMemcpyHostToDevice, b->stream));
+    OD_BCK(b, cudaMemcpyAsync(b->d_tasks, step.data(), sizeof(int2) * step.size(), cudaMemcpyHostToDevice, b->stream));
     if (!fk.empty())
         OD_BCK(b, cudaMemcpyAsync(b->d_tasks_f, fk.data(), sizeof(int2) * fk.size(), cudaMemcpyHostToDevice, b->stream));
     b->grid = (int)std::max(1ll, std::min<long long>((long long)batch_blocks_per_sm(b->ipt) * b->sms, b->T));
@@ -230,7 +227,7 @@ int od_batch_step(od_batch* b, int64_t n)
         b->gexec = nullptr;
         b->graph = nullptr;
         OD_BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-        const int lrc = launch_batch(b->ipt, b->grid, b->d_runs, b->d_tasks, b->phase_end, b->T, b->d_bc, b->d_done,
+        const int lrc = launch_batch(b->ipt, b->grid, b->d_runs, b->d_tasks, b->T, b->d_bc, b->d_done,
                                      (int)b->runs.size(), SPIN_LIMIT, 0, b->stream);
         cudaGraph_t g = nullptr;
         const cudaError_t e = cudaStreamEndCapture(b->stream, &g);
@@ -258,7 +255,7 @@ int od_batch_size(const od_batch* b) { return b ? (int)b->runs.size() : 0; }
 // forces-only mode (fresh counters per configuration)
 static int batch_tune_launch(od_batch* b, int grid)
 {
-    const int lrc = launch_batch(b->ipt, grid, b->d_runs, b->d_tasks_f, b->phase_end_f, b->T_f, b->d_bc_f,
+    const int lrc = launch_batch(b->ipt, grid, b->d_runs, b->d_tasks_f, b->T_f, b->d_bc_f,
                                  b->d_done_f, (int)b->runs.size(), SPIN_LIMIT, 1, b->stream);
     return lrc ? bfail(b, OD_ECUDA, "batch tune launch failed") : OD_OK;
 }

@@ -163,11 +163,11 @@ int od_tune(od_handle* h, int reps, double* ms, int* best_variant, int* best_upb
                 // the kick is timed too: it sums the ordered kernel's partial slots, or reads
                 // and clears the symmetric kernels' fixed-point sums
                 OD_LK(h, launch_forces(h->P, h->B, h->F, h->variant, h->stream));
-                OD_LK(h, launch_kick(h->P, h->B, h->F, 1, h->stream));
+                OD_LK(h, launch_kick(h->P, h->B, h->F, h->stream));
                 OD_CK(h, cudaEventRecord(h->ev[0], h->stream));
                 for (int r = 0; r < reps; ++r) {
                     OD_LK(h, launch_forces(h->P, h->B, h->F, h->variant, h->stream));
-                    OD_LK(h, launch_kick(h->P, h->B, h->F, 1, h->stream));
+                    OD_LK(h, launch_kick(h->P, h->B, h->F, h->stream));
                 }
                 OD_CK(h, cudaEventRecord(h->ev[1], h->stream));
                 OD_CK(h, cudaEventSynchronize(h->ev[1]));
@@ -187,11 +187,11 @@ int od_tune(od_handle* h, int reps, double* ms, int* best_variant, int* best_upb
             int rc = apply_force_config(h, timed[f].v, timed[f].g, timed[f].b);
             if (rc) return rc;
             OD_LK(h, launch_forces(h->P, h->B, h->F, h->variant, h->stream));
-            OD_LK(h, launch_kick(h->P, h->B, h->F, 1, h->stream));
+            OD_LK(h, launch_kick(h->P, h->B, h->F, h->stream));
             OD_CK(h, cudaEventRecord(h->ev[0], h->stream));
             for (int r = 0; r < reps; ++r) {
                 OD_LK(h, launch_forces(h->P, h->B, h->F, h->variant, h->stream));
-                OD_LK(h, launch_kick(h->P, h->B, h->F, 1, h->stream));
+                OD_LK(h, launch_kick(h->P, h->B, h->F, h->stream));
             }
             OD_CK(h, cudaEventRecord(h->ev[1], h->stream));
             OD_CK(h, cudaEventSynchronize(h->ev[1]));

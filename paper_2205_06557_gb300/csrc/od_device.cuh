@@ -682,10 +682,8 @@ __device__ __forceinline__ void push_scan_body(const Phys& P, const Bufs& B, int
     }
     // the step's number and the charges its ions feel, for the kick: the grain tail may change
     // the control block's before the kick reads them
-    if (B.felt) {
-        if (threadIdx.x == 32) B.felt->step = step;
-        if ((int)threadIdx.x < P.D) B.felt->Q[threadIdx.x] = C->Q[threadIdx.x];
-    }
+    if (threadIdx.x == 32) B.felt->step = step;
+    if ((int)threadIdx.x < P.D) B.felt->Q[threadIdx.x] = C->Q[threadIdx.x];
     __syncthreads();
     if (threadIdx.x == 0) {
         C->ev_step[9] += s_face[0];
@@ -801,22 +799,21 @@ __device__ __forceinline__ void grain_sums(const Phys& P, const Bufs& B, bool li
     }
 }
 
-// mode 0: after the push (second half kick + collisions); mode 1: forces only (creation
-// or a replaced ion state).  PRE (single runs' steps): the ion terms, the collision velocities
-// and the grain side have been computed beside the pair forces (Bufs::pre, coll_v; the step
-// number and the charges the ions feel are Bufs::felt's).
-template <int BT, int CP_WIDE = 8, bool PRE = false>
-__device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const ForceArgs& F, int mode, int blk)
+// STEP: a step's kick after the push (second half kick + collisions); the ion terms, the collision
+// velocities and the grain side have been computed beside the pair forces (Bufs::pre, coll_v;
+// the step number and the charges the ions feel are Bufs::felt's).  Otherwise forces only
+// (creation, a replaced ion state, tuning): accelerations and the grain side.
+template <int BT, int CP_WIDE = 8, bool STEP = false>
+__device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const ForceArgs& F, int blk)
 {
     __shared__ double s_Q[MAXD];
     Ctrl* C = B.ctrl;
-    const long long step = PRE ? B.felt->step : C->step;
-    const int buf = mode == 0 ? (int)((step + 1) & 1) : (int)(step & 1);
+    const long long step = STEP ? B.felt->step : C->step;
+    const int buf = STEP ? (int)((step + 1) & 1) : (int)(step & 1);
     const uint32_t sn = (uint32_t)(step + 1);
     const int i = blk * BT + threadIdx.x;
     const bool live = i < C->n_cur;
     const long long cap = B.cap;
-    const int lane = threadIdx.x & 31;
     const bool sym_sums = F.sym && !(P.flags & OD_F_NO_IONION);
     // every load that does not depend on another is issued first (one memory round trip):
     // position, velocity, id, the fixed-point pair sums, the ion terms, the grain charges
@@ -830,14 +827,12 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
         x = X[i];
         y = X[cap + i];
         z = X[2 * cap + i];
-        if (mode == 0) {
+        if (STEP) {
             const double* V = B.v[buf];
             vx = V[i];
             vy = V[cap + i];
             vz = V[2 * cap + i];
             id = B.id[buf][i];
-        }
-        if (PRE) {
             const double* T = B.pre;
             cx = __ldcg(T + i), cy = __ldcg(T + cap + i), cz = __ldcg(T + 2 * cap + i);
             bx = __ldcg(T + 3 * cap + i), by = __ldcg(T + 4 * cap + i), bz = __ldcg(T + 5 * cap + i);
@@ -851,12 +846,11 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
             qc = A[2 * F.psum_ld];
         }
     }
-    if ((int)threadIdx.x < P.D) s_Q[threadIdx.x] = PRE ? B.felt->Q[threadIdx.x] : C->Q[threadIdx.x];
+    if ((int)threadIdx.x < P.D) s_Q[threadIdx.x] = STEP ? B.felt->Q[threadIdx.x] : C->Q[threadIdx.x];
     __syncthreads();
-    int coll = 0;
     if (live) {
-        if (!PRE && P.cp_on) close_pairs_of<CP_WIDE>(P, B, buf, i, x, y, z, cx, cy, cz);
-        if (!PRE) ion_field(P, x, y, z, bx, by, bz);
+        if (!STEP && P.cp_on) close_pairs_of<CP_WIDE>(P, B, buf, i, x, y, z, cx, cy, cz);
+        if (!STEP) ion_field(P, x, y, z, bx, by, bz);
         float ax = 0.f, ay = 0.f, az = 0.f;
         if (!(P.flags & OD_F_NO_IONION)) {
             double px = 0.0, py = 0.0, pz = 0.0;  // pair sum in scaled units
@@ -928,7 +922,7 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
         }
         const float4 a = make_float4((float)((double)ax + bx), (float)((double)ay + by), (float)((double)az + bz), 0.f);
         B.acc[i] = a;
-        if (mode == 0) {
+        if (STEP) {
             double* V = B.v[buf];
             const double h = 0.5 * P.dt;
             vx += h * (double)a.x;
@@ -937,15 +931,10 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
             // Andersen collision with the neutrals: integer threshold on a Philox word
             const uint4 w = philox(P, id, sn, ST_COLL);
             if ((unsigned long long)w.x < P.Tcoll) {
-                if (mode == 0 && B.coll_v) {
-                    // drawn beside the pair forces (same stream of random numbers)
-                    vx = __ldcg(B.coll_v + i);
-                    vy = __ldcg(B.coll_v + cap + i);
-                    vz = __ldcg(B.coll_v + 2 * cap + i);
-                } else {
-                    collision_velocity(P, id, sn, vx, vy, vz);
-                }
-                coll = 1;
+                // drawn beside the pair forces
+                vx = __ldcg(B.coll_v + i);
+                vy = __ldcg(B.coll_v + cap + i);
+                vz = __ldcg(B.coll_v + 2 * cap + i);
             }
             if (P.flags & OD_F_FP32_STATE) vx = rnd32(vx), vy = rnd32(vy), vz = rnd32(vz);
             V[i] = vx;
@@ -963,10 +952,7 @@ __device__ __forceinline__ void kick_body(const Phys& P, const Bufs& B, const Fo
             F.psum[2 * F.psum_ld + e] = 0;
         }
     }
-    if (PRE) return;
-    const unsigned bc = __ballot_sync(0xffffffffu, coll);
-    if (lane == 0 && bc) atomicAdd(&C->ev_step[12], __popc(bc));
-    grain_sums<BT>(P, B, live, x, y, z, blk);
+    if (!STEP) grain_sums<BT>(P, B, live, x, y, z, blk);
 }
 
 // --------------------------------------------------------------- grain tail

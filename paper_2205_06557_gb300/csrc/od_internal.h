@@ -150,10 +150,10 @@ struct Bufs {
     Rem* rem;
     Inj* inj_ahead;  // [INJ_AHEAD] injection samples of the next step, computed during this one
     double* coll_v;  // [3][cap] neutral velocities of this step's colliding ions, computed beside the
-                     // pair forces (null: the kick draws them)
+                     // pair forces
     double* pre;   // [6][cap] the step's ion terms (close-pair correction, E_out and driving field),
-                   // computed beside the pair forces (single runs)
-    Felt* felt;    // null in a batch
+                   // computed beside the pair forces
+    Felt* felt;
     double* dpart; // grain partial sums [nb][MAXD][3]
     Ctrl* ctrl;
     long long cap;
@@ -204,12 +204,13 @@ struct BatchCtrl {
     int err;
 };
 
-constexpr int BATCH_TILE = 128;  // ions per scan / kick tile and threads per CTA of a batch
+constexpr int BATCH_TILE = 128;  // ions per scan / side / kick tile and threads per CTA of a batch
+// task kinds, in the order a step hands them out (the last only in tuning launches)
+enum BatchTask { BT_SCAN = 0, BT_PAIR = 1, BT_SIDE = 2, BT_TAIL = 3, BT_KICK = 4, BT_FORCES = 5 };
 ForceArgs batch_plan(int N, int ipt, int jc);
 int batch_blocks_per_sm(int ipt);
-int launch_batch(int ipt, int grid, const RunDesc* runs, const int2* tasks, int4 phase_end, long long T,
-                 BatchCtrl* bc, unsigned long long* done, int R, long long spin_limit, int tune,
-                 cudaStream_t s);
+int launch_batch(int ipt, int grid, const RunDesc* runs, const int2* tasks, long long T, BatchCtrl* bc,
+                 unsigned long long* done, int R, long long spin_limit, int tune, cudaStream_t s);
 
 // host launchers (od_kernels.cu)
 int launch_init_ions(const Phys& P, const Bufs& B, cudaStream_t s);
@@ -217,7 +218,7 @@ int launch_fpos(const Phys& P, const Bufs& B, int buf, cudaStream_t s);
 int launch_pad(const Phys& P, const Bufs& B, cudaStream_t s);
 int launch_push_scan(const Phys& P, const Bufs& B, cudaStream_t s);
 int launch_forces(const Phys& P, const Bufs& B, const ForceArgs& F, int variant, cudaStream_t s);
-int launch_kick(const Phys& P, const Bufs& B, const ForceArgs& F, int mode, cudaStream_t s);
+int launch_kick(const Phys& P, const Bufs& B, const ForceArgs& F, cudaStream_t s);  // forces only
 int launch_cp_bump(const Bufs& B, cudaStream_t s);  // advance the close-pair list epoch
 int launch_kick_step(const Phys& P, const Bufs& B, const ForceArgs& F, cudaStream_t s);
 // beside a step's pair forces: the next step's first INJ_AHEAD injection samples, the ion

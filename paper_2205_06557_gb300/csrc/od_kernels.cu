@@ -293,16 +293,16 @@ __global__ void __launch_bounds__(BT) k_push_scan(Phys P, Bufs B, int n_tiles, d
 // A step's kick: the pair forces, the precomputed ion terms and the grain Coulomb force
 __global__ void __launch_bounds__(KICK_BT) k_kick_step(Phys P, Bufs B, ForceArgs F)
 {
-    kick_body<KICK_BT, 8, true>(P, B, F, 0, blockIdx.x);
+    kick_body<KICK_BT, 8, true>(P, B, F, blockIdx.x);
 }
 
-// The whole kick, then the grain tail in the last block to finish (the grain update reads every
+// Accelerations and grain sums, then the grain tail in the last block to finish (the grain update reads every
 // block's sums): force evaluations outside the steps
 template <int BT>
-__global__ void __launch_bounds__(BT) k_kick(Phys P, Bufs B, ForceArgs F, int mode)
+__global__ void __launch_bounds__(BT) k_kick(Phys P, Bufs B, ForceArgs F)
 {
     __shared__ int s_last;
-    kick_body<BT>(P, B, F, mode, blockIdx.x);
+    kick_body<BT>(P, B, F, blockIdx.x);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) s_last = atomicAdd(&B.ctrl->kick_done, 1u) == gridDim.x - 1;
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(BT) k_kick(Phys P, Bufs B, ForceArgs F, int mo
     if (!s_last) return;
     __threadfence();
     if (threadIdx.x == 0) B.ctrl->kick_done = 0u;
-    dust_body(P, B, (int)gridDim.x, mode);
+    dust_body(P, B, (int)gridDim.x, 1);
 }
 
 
@@ -655,10 +655,10 @@ int launch_forces(const Phys& P, const Bufs& B, const ForceArgs& F, int v, cudaS
     return (int)cudaErrorInvalidValue;
 }
 
-int launch_kick(const Phys& P, const Bufs& B, const ForceArgs& F, int mode, cudaStream_t s)
+int launch_kick(const Phys& P, const Bufs& B, const ForceArgs& F, cudaStream_t s)
 {
     if (P.N == 0) return 0;
-    k_kick<KICK_BT><<<(P.N + KICK_BT - 1) / KICK_BT, KICK_BT, 0, s>>>(P, B, F, mode);
+    k_kick<KICK_BT><<<(P.N + KICK_BT - 1) / KICK_BT, KICK_BT, 0, s>>>(P, B, F);
     return ck(cudaGetLastError());
 }
 
