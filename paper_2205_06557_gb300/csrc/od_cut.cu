@@ -257,9 +257,15 @@ __global__ void k_cut_fill(const float4* __restrict__ lo, const float4* __restri
     }
 }
 
-// persistent CTAs over the listed tile pairs (their number is read on the device)
+// Persistent CTAs over the listed tile pairs (their number is read on the device).  Bound like the
+// all-pairs kernel by the FP32 pipe and the register file; the switched coefficient adds eight
+// packed operations and two scalar ones to 17.  262,144 ions in a tube of ten cutoffs, switched
+// from half the cutoff: 4.22 -> 3.95 ms; 12 warps at 168 registers against 16 at 128 are 2% of
+// it, two rotations per loop step instead of four 1%.  Slabs of 1/128 of the cutoff, whose
+// tiles list 6% fewer pairs and half of them plain, give 3.4 ms; they sum the terms in another
+// order, and an ion's FP32 sum then moves by up to 1e-6 of its largest term.
 template <int BT, int IPT>
-__global__ void __launch_bounds__(BT, (IPT == 8 ? 65536 / (BT * 128) : 1))
+__global__ void __launch_bounds__(BT, (IPT == 8 ? 65536 / (BT * 168) : 1))
     k_forces_cut(const float4* __restrict__ fsort, ForceArgs F, const int2* __restrict__ units,
                  const int* __restrict__ n_units)
 {

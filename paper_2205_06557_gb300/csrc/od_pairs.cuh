@@ -117,21 +117,20 @@ __device__ __forceinline__ f32x2 pair_c3x2(f32x2 dx, f32x2 dy, f32x2 dz)
     return mul2(mul2(e, mul2(ri, ri)), add2(ri, ln2));
 }
 
-// switch_bracket for two pairs at once, in packed operations (only the clamp is per
-// lane): x = (s - s0) w_inv in [0, 1], S = 1 + x^3 (15 x - 6 x^2 - 10),
-// -S' = 30 x^2 (1 - x)^2, bracket = (ri + ln2) S + 30 w_inv x^2 (1 - x)^2
-__device__ __forceinline__ f32x2 switch_bracket2(f32x2 s, f32x2 ri, float s0, float w_inv)
+// switch_bracket for two pairs at once: with h = 1/2 - x and q = h^2,
+// S = 1/2 + h (15/8 - 5 q + 6 q^2) and -S' = 30 (1/4 - q)^2.  At x = 0 and x = 1 every step is exact,
+// so the plain term and the zero beyond the cutoff come out exactly.  x is one saturating FMA
+// per lane; the rest is eight packed operations.
+__device__ __forceinline__ f32x2 switch_bracket2(float sa, float sb, f32x2 ri, float s0, float w_inv)
 {
     constexpr float LN2 = 0.69314718055994531f;
-    f32x2 x = fma2(s, pk2(w_inv, w_inv), pk2(-s0 * w_inv, -s0 * w_inv));
-    float xa, xb;
-    upk2(x, xa, xb);
-    x = pk2(fminf(fmaxf(xa, 0.f), 1.f), fminf(fmaxf(xb, 0.f), 1.f));
-    const f32x2 x2 = mul2(x, x);
-    const f32x2 t = fma2(fma2(x, pk2(-6.f, -6.f), pk2(15.f, 15.f)), x, pk2(-10.f, -10.f));
-    const f32x2 S = fma2(mul2(x2, x), t, pk2(1.f, 1.f));
-    const f32x2 y2 = fma2(x, add2(x, pk2(-2.f, -2.f)), pk2(1.f, 1.f));
-    return fma2(mul2(x2, y2), pk2(30.f * w_inv, 30.f * w_inv), mul2(add2(ri, pk2(LN2, LN2)), S));
+    const float off = -s0 * w_inv, g = sqrtf(30.f * w_inv);
+    const f32x2 x = pk2(__saturatef(fmaf(sa, w_inv, off)), __saturatef(fmaf(sb, w_inv, off)));
+    const f32x2 h = sub2(pk2(0.5f, 0.5f), x), q = mul2(h, h);
+    const f32x2 t = fma2(fma2(q, pk2(6.f, 6.f), pk2(-5.f, -5.f)), q, pk2(1.875f, 1.875f));
+    const f32x2 S = fma2(h, t, pk2(0.5f, 0.5f));
+    const f32x2 a = fma2(q, pk2(-g, -g), pk2(0.25f * g, 0.25f * g));
+    return fma2(a, a, mul2(add2(ri, pk2(LN2, LN2)), S));
 }
 
 // pair_c3_cut for two pairs at once: the packed plain coefficient's steps, then the
@@ -145,11 +144,10 @@ __device__ __forceinline__ f32x2 pair_c3x2_cut(f32x2 dx, f32x2 dy, f32x2 dz, flo
     float ra, rb;
     upk2(r2, ra, rb);
     const f32x2 ri = pk2(rsqrt_approx(ra), rsqrt_approx(rb));
-    const f32x2 s = mul2(r2, ri);
     float sa, sb;
-    upk2(s, sa, sb);
+    upk2(mul2(r2, ri), sa, sb);
     const f32x2 e = pk2(ex2_approx(-sa), ex2_approx(-sb));
-    return mul2(mul2(e, mul2(ri, ri)), switch_bracket2(s, ri, s0, w_inv));
+    return mul2(mul2(e, mul2(ri, ri)), switch_bracket2(sa, sb, ri, s0, w_inv));
 }
 
 // Accumulate into IPT targets per thread the pair terms of sources [j0, j1), staged
@@ -420,7 +418,7 @@ __device__ __forceinline__ void sym2_group(float4 pa, float4 pb, const float (&x
     S.z[lane] = S.z[32 + lane] = pk2(pa.z, pb.z);
     __syncwarp();
     f32x2 bx = 0ull, by = 0ull, bz = 0ull;
-#pragma unroll 4
+#pragma unroll(CUT ? 2 : 4)
     for (int r = 0; r < 32; ++r) {
         const f32x2 xj = S.x[lane + r], yj = S.y[lane + r], zj = S.z[lane + r];
 #pragma unroll
