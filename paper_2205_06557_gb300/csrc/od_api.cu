@@ -518,11 +518,27 @@ int ensure_part(od_handle* h)
 {
     const long long need = (long long)h->F.W * h->F.n_pad;
     if (need == 0) return OD_OK;  // symmetric kernels: fixed-point accumulators only
-    if (need <= h->part_cap) return OD_OK;
-    if (h->B.part) cudaFree(h->B.part);
-    h->B.part = nullptr;
-    OD_CK(h, cudaMalloc(&h->B.part, sizeof(float4) * std::max(need, 1ll)));
-    h->part_cap = need;
+    if (need > h->part_cap) {
+        if (h->B.part) cudaFree(h->B.part);
+        h->B.part = nullptr;
+        OD_CK(h, cudaMalloc(&h->B.part, sizeof(float4) * std::max(need, 1ll)));
+        h->part_cap = need;
+    }
+    // block sums (12 bytes per ion and block of 128 ions); without the memory for them the
+    // ordered kernel makes the same sums
+    if (h->batch_member || (h->P.flags & OD_F_FP64_PAIRS) || !wave_sums(h->F, h->variant)) return OD_OK;
+    const long long nblk = 3ll * (h->F.n_pad / 128) * h->F.n_pad;
+    if (nblk > h->blk_cap) {
+        cudaFree(h->d_blk);
+        h->d_blk = nullptr;
+        h->blk_cap = 0;
+        if (cudaMalloc(&h->d_blk, sizeof(float) * nblk) != cudaSuccess) {
+            cudaGetLastError();
+            return OD_OK;
+        }
+        h->blk_cap = nblk;
+    }
+    h->F.blk = h->d_blk;
     return OD_OK;
 }
 
@@ -761,6 +777,7 @@ void free_all(od_handle* h)
     cudaFree(h->B.ctrl);
     cudaFree(h->d_stats);
     cudaFree(h->d_sched);
+    cudaFree(h->d_blk);
     cudaFree(h->d_vtab);
     cudaFree(h->d_series);
     cudaFree(h->d_evseries);

@@ -45,6 +45,8 @@ struct od_handle {
     long long cap = 0;       // ion capacity
     long long npad_cap = 0;  // fpos capacity
     long long part_cap = 0;  // partial-sum capacity (float4)
+    float* d_blk = nullptr;   // block sums (ForceArgs::blk)
+    long long blk_cap = 0;    // floats
     long long nb_cap = 0;    // kick blocks capacity
     long long scan_tiles_cap = 0;  // scan tile status words (tiles of the smaller of the single-run and batch scan)
     long long host_step = 0;

@@ -183,6 +183,9 @@ struct ForceArgs {
     // dynamic unit queue of the packed symmetric and cutoff kernels: [0] next unit,
     // [1] CTAs finished (both zero between launches)
     unsigned long long* sched;
+    // block sums [n_pad / 128][3][n_pad] of the ordered kernel with 128-source blocks made from
+    // unordered pairs (null: the ordered kernel itself)
+    float* blk;
     // live ion count (device; the plan covers the capacity under the flux rule), or null
     const int* n_live;
 };
@@ -218,6 +221,8 @@ int launch_fpos(const Phys& P, const Bufs& B, int buf, cudaStream_t s);
 int launch_pad(const Phys& P, const Bufs& B, cudaStream_t s);
 int launch_push_scan(const Phys& P, const Bufs& B, cudaStream_t s);
 int launch_forces(const Phys& P, const Bufs& B, const ForceArgs& F, int variant, cudaStream_t s);
+int launch_forces_wave(const Bufs& B, const ForceArgs& F, int variant, cudaStream_t s);
+bool wave_sums(const ForceArgs& F, int variant);  // whether launch_forces can take F.blk
 int launch_kick(const Phys& P, const Bufs& B, const ForceArgs& F, cudaStream_t s);  // forces only
 int launch_cp_bump(const Bufs& B, cudaStream_t s);  // advance the close-pair list epoch
 int launch_kick_step(const Phys& P, const Bufs& B, const ForceArgs& F, cudaStream_t s);
