@@ -407,6 +407,21 @@ __device__ void close_pair_corr(const unsigned long long* __restrict__ head, con
 // split into chunks of at most 64, each drawn by inversion (summing e^-l l^x / x! in
 // increasing x until the sum reaches one uniform); uniform j of the step is word j mod 4
 // of the Philox block with counter (j / 4, 0, sn, ST_INJ_N).  FP64 throughout.
+__device__ __forceinline__ int poisson_chunk(const Phys& P, uint32_t sn, int j, double l)
+{
+    const uint4 w = philox(P, (unsigned long long)(j >> 2), sn, ST_INJ_N);
+    const uint32_t wj = (j & 3) == 0 ? w.x : (j & 3) == 1 ? w.y : (j & 3) == 2 ? w.z : w.w;
+    const double U = unif(wj);
+    double pr = exp(-l), F = pr;
+    int x = 0;
+    while (U > F && x < 100000) {
+        ++x;
+        pr = pr * (l / (double)x);
+        F += pr;
+    }
+    return x;
+}
+
 __device__ __forceinline__ int poisson_injections(const Phys& P, uint32_t sn)
 {
     double rem = P.inj_lambda;
@@ -414,19 +429,19 @@ __device__ __forceinline__ int poisson_injections(const Phys& P, uint32_t sn)
     for (int j = 0; rem > 0.0; ++j) {
         const double l = rem > 64.0 ? 64.0 : rem;
         rem -= l;
-        const uint4 w = philox(P, (unsigned long long)(j >> 2), sn, ST_INJ_N);
-        const uint32_t wj = (j & 3) == 0 ? w.x : (j & 3) == 1 ? w.y : (j & 3) == 2 ? w.z : w.w;
-        const double U = unif(wj);
-        double pr = exp(-l), F = pr;
-        int x = 0;
-        while (U > F && x < 100000) {
-            ++x;
-            pr = pr * (l / (double)x);
-            F += pr;
-        }
-        k += x;
+        k += poisson_chunk(P, sn, j, l);
     }
     return k;
+}
+
+// the same number drawn by a warp, one chunk per lane at a time (lam - 64 j is exact, as the
+// repeated subtraction is)
+__device__ __forceinline__ int poisson_injections_warp(const Phys& P, uint32_t sn)
+{
+    int k = 0;
+    for (int j = threadIdx.x & 31; P.inj_lambda - 64.0 * j > 0.0; j += 32)
+        k += poisson_chunk(P, sn, j, fmin(P.inj_lambda - 64.0 * j, 64.0));
+    return __reduce_add_sync(0xffffffffu, k);
 }
 
 // ------------------------------------------------- push + scan + compaction
@@ -641,7 +656,7 @@ __device__ __forceinline__ void push_scan_body(const Phys& P, const Bufs& B, int
         s_m = m;
         // injections: one per removed ion, or a Poisson number from the fluxes (clamped
         // to the capacity, which reports an overflow)
-        int k = flux ? poisson_injections(P, sn) : m;
+        int k = !flux ? m : C->ahead_sn == (long long)sn ? C->ahead_kin : poisson_injections(P, sn);
         if (n_live - m + k > P.N) {
             k = P.N - (n_live - m);
             atomicOr(&C->err, ERR_OVERFLOW);

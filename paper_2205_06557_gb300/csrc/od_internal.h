@@ -60,7 +60,7 @@ struct Ctrl {
     long long ahead_sn;
     long long ahead_req_sn;       // the step the next samples are for (set by the scan's last tile)
     int ahead_want;               // how many to draw (the scan's estimate of the next step's need)
-    int ahead_pad;
+    int ahead_kin;                // flux rule: how many ions enter in step ahead_sn
     double* series;               // [cap][MAXD][REC]
     int* evseries;                // [cap][EV]
     long long series_cap;
