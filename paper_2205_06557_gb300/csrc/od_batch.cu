@@ -5,17 +5,19 @@
 // target tile x one source chunk (or tile pairs); side tiles of 128 ions (the ion terms and
 // the grain sums, which need the positions but not the pair forces); a grain tail; kick tiles.
 // A persistent grid of at most the resident number of CTAs takes tasks from a global
-// counter, all scan tiles first, then all pair units, side tiles, tails and kick tiles (runs
-// in order inside each kind), so the side tiles and tails fill the CTAs that run out of pair
-// units while others still work on theirs.  A task first waits until the counters of the
-// kinds it depends on (of its run) reach their targets: pair units and side tiles for the
-// scan, the tail for the side tiles, the kick for the pair units and the side tiles; every
-// task waited for was handed out earlier to a CTA that is running, so the waits end (and
-// each is bounded anyway: it gives up after spin_limit polls and sets an error).
+// counter: the runs' pair units one run after the other, each run's scan tiles well ahead of them
+// and its side tiles between them, then all tails and kick tiles.  A task first waits until the
+// counters of the kinds it depends on (of its run) reach their targets: pair units and side
+// tiles for the scan, the tail for the side tiles, the kick for the pair units and the side
+// tiles; every task waited for was handed out earlier to a CTA that is running, so the waits
+// end (and each is bounded anyway: it gives up after spin_limit polls and sets an error).
 // The counters only grow (target = (batch step + 1) x tasks of the kind), so nothing
 // is reset between launches; the last CTA to leave advances the batch step.
-// 48 runs of 2,171 ions (tile pairs of 256 ions): 195 us per step (cold caches); 223 with the ion terms and
-// grain sums inside the kick tiles and one tail per run after them.
+// What bounds it: the latency of a step's chain (scan, pair units, kick) and, between, the FP32 pipe
+// for the pair units and the FP64 pipe for the rest, which is why the two are mixed.  48 runs of
+// 2,171 ions (tile pairs of 256 ions), per step: 223 us with the ion terms and grain sums
+// inside the kick tiles, 198 with side tiles of their own after all pair units, 181 with the
+// side tiles between the pair units and polls at most 256 ns apart.  32 runs of 6,283: 578 -> 553.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -85,7 +87,7 @@ __device__ __forceinline__ void wait_count(const unsigned long long* cnt, unsign
                 break;
             }
             __nanosleep(ns);
-            if (ns < 2048) ns *= 2;
+            if (ns < 256) ns *= 2;
         }
     }
     __syncthreads();

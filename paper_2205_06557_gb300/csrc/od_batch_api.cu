@@ -59,10 +59,6 @@ int batch_build(od_batch* b)
 {
     const int R = (int)b->runs.size();
     std::vector<RunDesc> desc(R);
-    std::vector<int2> all[BT_FORCES + 1];  // tasks by kind
-    auto add = [&](int kind, int r, long long n) {
-        for (long long i = 0; i < n; ++i) all[kind].push_back(make_int2(kind << 28 | r, (int)i));
-    };
     for (int r = 0; r < R; ++r) {
         od_handle* h = b->runs[r];
         h->F = batch_plan(h->P.N, b->ipt, b->jc);
@@ -80,16 +76,35 @@ int batch_build(od_batch* b)
         desc[r].nK = desc[r].nA;
         if (desc[r].nA > h->scan_tiles_cap || desc[r].nK > h->nb_cap)
             return bfail(b, OD_EINVAL, "batch: run " + std::to_string(r) + " has more scan or kick tiles than its buffers");
-        add(BT_SCAN, r, desc[r].nA);
-        add(BT_PAIR, r, h->F.U);
-        add(BT_SIDE, r, desc[r].nK);
-        add(BT_TAIL, r, 1);
-        add(BT_KICK, r, desc[r].nK);
-        add(BT_FORCES, r, desc[r].nK);
     }
-    std::vector<int2> step, fk(all[BT_PAIR]);
-    for (int k = BT_SCAN; k <= BT_KICK; ++k) step.insert(step.end(), all[k].begin(), all[k].end());
-    fk.insert(fk.end(), all[BT_FORCES].begin(), all[BT_FORCES].end());
+    // The step's tasks in the order they are handed out; a task comes after all it waits for.
+    // The pair units are the FP32 work and the rest is FP64 (a third of the step's cycles on
+    // that pipe), so the side tiles are spread along their run's pair units and the scans
+    // come four grids' worth of pair units ahead of their run's first one.  Tails and kicks
+    // stay at the end: a grid or three behind their run's last pair unit they still wait for
+    // it too often (632 and 563 us instead of 555 per step of 32 runs of 6,283 ions).
+    const long long ctas = (long long)batch_blocks_per_sm(b->ipt) * b->sms;
+    std::vector<int2> step, fk;
+    auto add = [](std::vector<int2>& v, int kind, int r, long long i0, long long i1) {
+        for (long long i = i0; i < i1; ++i) v.push_back(make_int2(kind << 28 | r, (int)i));
+    };
+    int scans = 0;
+    long long pos = 0, scan_at = 0;  // pair units handed out; those before run `scans`' first one
+    for (int r = 0; r < R; ++r) {
+        const long long U = desc[r].F.U, nK = desc[r].nK;
+        for (long long u = 0; u < std::max(U, 1ll); ++u) {
+            for (; scans < R && (scans <= r || scan_at <= pos + 4 * ctas); ++scans) {
+                add(step, BT_SCAN, scans, 0, desc[scans].nA);
+                scan_at += desc[scans].F.U;
+            }
+            if (u < U) add(step, BT_PAIR, r, u, u + 1), ++pos;
+            add(step, BT_SIDE, r, u * nK / std::max(U, 1ll), (u + 1) * nK / std::max(U, 1ll));
+        }
+    }
+    for (int r = 0; r < R; ++r) add(step, BT_TAIL, r, 0, 1);
+    for (int r = 0; r < R; ++r) add(step, BT_KICK, r, 0, desc[r].nK);
+    for (int r = 0; r < R; ++r) add(fk, BT_PAIR, r, 0, desc[r].F.U);
+    for (int r = 0; r < R; ++r) add(fk, BT_FORCES, r, 0, desc[r].nK);
     b->T = (long long)step.size();
     b->T_f = (long long)fk.size();
     cudaFree(b->d_runs);
@@ -104,7 +119,7 @@ int batch_build(od_batch* b)
     OD_BCK(b, cudaMemcpyAsync(b->d_tasks, step.data(), sizeof(int2) * step.size(), cudaMemcpyHostToDevice, b->stream));
     if (!fk.empty())
         OD_BCK(b, cudaMemcpyAsync(b->d_tasks_f, fk.data(), sizeof(int2) * fk.size(), cudaMemcpyHostToDevice, b->stream));
-    b->grid = (int)std::max(1ll, std::min<long long>((long long)batch_blocks_per_sm(b->ipt) * b->sms, b->T));
+    b->grid = (int)std::max(1ll, std::min<long long>(ctas, b->T));
     OD_BCK(b, cudaStreamSynchronize(b->stream));
     b->graph_ok = false;
     return OD_OK;
