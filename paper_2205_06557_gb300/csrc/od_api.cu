@@ -647,12 +647,16 @@ int launch_density(od_handle* h)
     return OD_OK;
 }
 
-// what runs beside the pair forces, on three more streams (forked after the scan): the ion
+// The pair forces, and what runs beside them on three more streams (forked after the scan): the ion
 // terms the kick adds (joined by join_terms before it), the grain side and the next step's
-// injection samples (joined by join_rest before the step ends)
-int fork_beside(od_handle* h)
+// injection samples (joined by join_rest before the step ends).  The pair forces are
+// launched first: their CTAs then spread evenly over the SMs and the small kernels fill in.  The
+// other way round they went where the small kernels left room (whole steps of 4,500, 8,000,
+// 20,000 and 32,000 ions: 62.6, 84.5, 199 and 408 us; pair forces first 46.0, 72.9, 189 and 396).
+int pairs_and_beside(od_handle* h)
 {
     OD_CK(h, cudaEventRecord(h->ev_fork, h->stream));
+    OD_LK(h, launch_pairs(h, 1));
     for (int k = 0; k < 3; ++k) OD_CK(h, cudaStreamWaitEvent(h->aux[k], h->ev_fork, 0));
     OD_LK(h, launch_ion_terms(h->P, h->B, h->aux[0]));
     OD_LK(h, launch_grains(h->P, h->B, h->aux[1]));
@@ -677,8 +681,7 @@ int launch_step(od_handle* h)
 {
     int rc;
     OD_LK(h, launch_push_scan(h->P, h->B, h->stream));
-    if ((rc = fork_beside(h))) return rc;
-    OD_LK(h, launch_pairs(h, 1));
+    if ((rc = pairs_and_beside(h))) return rc;
     if ((rc = join_terms(h))) return rc;
     OD_LK(h, launch_kick_step(h->P, h->B, h->F, h->stream));
     if ((rc = join_rest(h))) return rc;
@@ -1034,8 +1037,7 @@ int od_step(od_handle* h, int64_t n)
                 OD_CK(h, cudaEventRecord(e[0], h->stream));
                 OD_LK(h, launch_push_scan(h->P, h->B, h->stream));
                 OD_CK(h, cudaEventRecord(e[1], h->stream));
-                if ((rc = fork_beside(h))) return rc;
-                OD_LK(h, launch_pairs(h, 1));
+                if ((rc = pairs_and_beside(h))) return rc;
                 OD_CK(h, cudaEventRecord(e[2], h->stream));
                 if ((rc = join_terms(h))) return rc;
                 OD_LK(h, launch_kick_step(h->P, h->B, h->F, h->stream));

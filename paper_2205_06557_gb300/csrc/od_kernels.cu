@@ -4,7 +4,8 @@
 //   k_push_scan  first half kick + drift (velocity Verlet), absorption / outflow test,
 //                single-pass decoupled-look-back scan of the removal flags, stable
 //                compaction into the other state buffer, and 1:1 re-injection (App. B)
-//   k_forces*    all-pairs Yukawa ion-ion forces in FP32; beside them, on three more streams:
+//   k_forces*    all-pairs Yukawa ion-ion forces in FP32 (k_forces_wave: od_wave.cu); beside
+//                them, on three more streams:
 //                  k_ion_terms     close-pair correction, E_out (App. A) and E_ext on the ions,
 //                                  collision velocities
 //                  k_grains        the grain-side Yukawa sums of Eq. 1 (FP64); its last block runs

@@ -1,4 +1,4 @@
-// The ordered kernel's block sums from half the pair terms (10,241 to 32,768 ions).
+// The ordered kernel's block sums from half the pair terms (7,681 to 32,768 padded ions).
 //
 // k_forces<128, IPT> sums each target's terms over one block of 128 sources after another, every
 // block from zero in ascending source order.  This kernel makes the same block sums, bit for
@@ -194,12 +194,12 @@ __global__ void __launch_bounds__(WAVE_TI) k_fold_blocks(float4* __restrict__ pa
 // The ordered kernel stays where the wave's units (one warp for 41 us when alone on its scheduler)
 // are too few to fill the chip, and above 32,768 ions, where the block sums (12 n^2 / 128 bytes)
 // outgrow L2 and the symmetric kernels with fixed-point sums are the default anyway.
-// Pair sums of a step, ordered and wave (with the fold): 8,000 ions 52 and 50 us, 9,000 72 and
-// 71, 10,000 72 and 71, 11,000 82 and 72, 12,000 96 and 72, 16,000 160 and 121, 20,000 235 and
-// 171, 26,000 396 and 253, 32,768 601 and 408.
+// Whole steps, ordered and wave (with the fold): 6,000 ions 53 and 64 us, 7,000 61 and 66, 8,000
+// 73 and 69, 9,000 93 and 88, 12,000 117 and 90, 16,000 181 and 139, 20,000 255 and 189, 32,000
+// 612 and 396; the pair sums alone at 20,000 235 and 171, at 32,768 601 and 408.
 bool wave_sums(const ForceArgs& F, int v)
 {
-    constexpr int MIN_PAD = 10240, MAX_PAD = 32768;
+    constexpr int MIN_PAD = 7680, MAX_PAD = 32768;
     return !F.sym && !F.cut && v >= 0 && v < num_force_variants() && force_variant(v).BT == WAVE_B &&
            F.TI == WAVE_TI && F.n_pad > MIN_PAD && F.n_pad <= MAX_PAD;
 }

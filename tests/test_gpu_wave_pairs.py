@@ -1,4 +1,4 @@
-"""The ordered kernel's block sums made from unordered pairs (variant k_forces<128,2>, 10,241 to 32,768
+"""The ordered kernel's block sums made from unordered pairs (variant k_forces<128,2>, 7,681 to 32,768
 padded ions) at the edges of that range, with ragged last tiles and other plans, against an FP64 sum of
 the same positions: per ion within 1e-5 of the sum of the term magnitudes (the bar of the
 injected-state force tests), and the same bits from a repeated evaluation."""
@@ -13,7 +13,7 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,upb,bps", [(10240, 8, 0), (10241, 8, 0), (12032, 1, 0), (12033, 64, 2), (20011, 8, 0),
+@pytest.mark.parametrize("n,upb,bps", [(7680, 8, 0), (7681, 8, 0), (10241, 8, 0), (12032, 1, 0), (12033, 64, 2), (20011, 8, 0),
                                        (20011, 1000, 1), (32768, 8, 0), (32769, 8, 0)])
 def test_wave_accelerations_match_fp64(n, upb, bps):
     import paper_2205_06557_gb300 as od
