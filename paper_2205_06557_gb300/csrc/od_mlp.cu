@@ -27,7 +27,7 @@
 // Measured against the layer-by-layer kernels on the same engine (calls through the C ABI with
 // host arrays): forward of 16,384 samples 2,330 -> 260 us (kernels 510 -> 144 us; the rest was
 // host repacking); loss and gradients of 128 samples 605 -> 160 us (39 launches -> 4, of which
-// five serial column sums of 61 us), of 4,096 samples 10.7 -> 0.41 ms.
+// five serial column sums of 61 us), of 4,096 samples 10.7 -> 0.51 ms.
 //
 // Every wait is bounded: one that runs out sets bit 1 of *err and ends the CTA's work; loads in
 // flight are waited for (again bounded) and the tensor memory is freed.
@@ -829,12 +829,14 @@ int launch_forward_backward(const FusedMaps& M, const FusedArgs& A, int sms, int
 }
 
 // Row ranges: enough CTAs for the chip.  The tensor memory accumulator rounds towards zero, which
-// takes ~1e-9 of a sum per row off a chain; beyond 16,384 rows only two ranges, so that the
-// gradients stay within 2e-5 of those of a single chain (4,096 samples: 1.7e-5; thirteen ranges,
-// more exact, 3.2e-5).
+// takes ~1e-9 of a sum per row off a chain, so gradients summed over ranges move away from those
+// of a single chain as the rows grow (they get more exact).  They stay within 1.5e-5 of it: sms / 11
+// ranges up to 12,800 rows (1,600 samples: 1.4e-5; 2,048: 1.7e-5), two up to 20,480 (2,400
+// samples: 1.35e-5; 4,096: 2.1e-5), one beyond (4,096 samples, loss and gradients: 511 us
+// against 410 with two ranges).
 int grad_splits(int rows, int sms)
 {
-    const int nch = (rows + 63) / 64, want = rows > 16384 ? 2 : sms / W_TILES;
+    const int nch = (rows + 63) / 64, want = rows > 20480 ? 1 : rows > 12800 ? 2 : sms / W_TILES;
     return nch < want ? nch : want < 1 ? 1 : want;
 }
 

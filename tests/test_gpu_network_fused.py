@@ -11,7 +11,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("B", [1, 15, 16, 17, 129, 2049])  # less than a tile .. two ranges of rows
+@pytest.mark.parametrize("B", [1, 15, 16, 17, 129, 2049, 2600])  # less than a tile .. two ranges of rows, one
 def test_fused_kernels_agree_with_the_layer_by_layer_engine(B):
     import paper_2205_06557_gb300 as od
 
