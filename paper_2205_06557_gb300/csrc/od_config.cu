@@ -216,6 +216,13 @@ int od_tune(od_handle* h, int reps, double* ms, int* best_variant, int* best_upb
         h->part_cap = 0;
         if ((rc = ensure_part(h))) return rc;
     }
+    // and the block sums, if the chosen kernel makes none
+    if (h->d_blk && !h->F.blk) {
+        OD_CK(h, cudaStreamSynchronize(h->stream));
+        cudaFree(h->d_blk);
+        h->d_blk = nullptr;
+        h->blk_cap = 0;
+    }
     // the accelerations and partial sums left by the timing belong to other kernels:
     // evaluate the current state again with the chosen one
     if ((rc = force_eval(h))) return rc;
