@@ -840,6 +840,13 @@ int grad_splits(int rows, int sms)
     return nch < want ? nch : want < 1 ? 1 : want;
 }
 
+// The ranges fall as the rows grow, so a small batch may need more of them than a full one.
+int max_grad_splits(int max_rows, int sms)
+{
+    const int nch = (max_rows + 63) / 64, most = sms / W_TILES > 2 ? sms / W_TILES : 2;
+    return nch < most ? nch : most;
+}
+
 int launch_weight_grads(const GradMaps& M, float* part, int rows, int splits, int* err, cudaStream_t s)
 {
     const cudaError_t e = cudaFuncSetAttribute(k_weight_grads, cudaFuncAttributeMaxDynamicSharedMemorySize, W_SMEM);

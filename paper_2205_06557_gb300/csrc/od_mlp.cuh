@@ -58,6 +58,7 @@ int launch_forward_backward(const FusedMaps& M, const FusedArgs& A, int sms, int
 // weight gradients over rows (split over CTAs into partial vectors part[splits][N_PARAMS]),
 // then the whole gradient vector from the partials
 int grad_splits(int rows, int sms);
+int max_grad_splits(int max_rows, int sms);  // at least grad_splits of any rows up to max_rows
 int launch_weight_grads(const GradMaps& M, float* part, int rows, int splits, int* err, cudaStream_t s);
 int launch_grad_reduce(const float* part, int splits, const float* dbias, int bias_rows, float* grad, cudaStream_t s);
 

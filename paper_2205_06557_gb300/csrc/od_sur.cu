@@ -289,6 +289,7 @@ struct SurOut {
 
 struct od_sur {
     int maxB = 0, sms = 0;
+    int splits_cap = 0;  // partial gradients (ranges of rows) `part` holds
     Layer L[5];
     float *p = nullptr, *g = nullptr, *am = nullptr, *av = nullptr;  // parameters, gradients, Adam moments
     __nv_bfloat16 *wb = nullptr, *wt = nullptr;
@@ -524,7 +525,7 @@ int run_gradients(od_sur* s, int Bn, const float* mask_host)
         mlp::FusedArgs A = fused_args(s, Bn);
         A.y = nullptr;
         A.inv_count = inv;
-        const int splits = mlp::grad_splits(rows, s->sms);
+        const int splits = std::min(mlp::grad_splits(rows, s->sms), s->splits_cap);
         int ctas = 0;
         if ((e = mlp::launch_forward_backward(s->fmaps, A, s->sms, &ctas, s->stream)) ||
             (e = mlp::launch_weight_grads(s->gmaps, s->part, rows, splits, &s->d_out->err, s->stream)) ||
@@ -574,7 +575,8 @@ int od_sur_create(int max_batch, uint64_t seed, void* stream, od_sur** out)
     mb((void**)&s->y, 4 * M * OUTR);
     mb((void**)&s->rowl, 4 * M);
     mb((void**)&s->dbias, sizeof(float) * mlp::QUADS * mlp::BIAS_LD * (size_t)s->sms);
-    mb((void**)&s->part, sizeof(float) * mlp::N_PARAMS * (size_t)mlp::grad_splits((int)std::min(M, 16384ll), s->sms));
+    s->splits_cap = mlp::max_grad_splits((int)M, s->sms);
+    mb((void**)&s->part, sizeof(float) * mlp::N_PARAMS * (size_t)s->splits_cap);
     mb((void**)&s->acts.x0, 2 * M * K0);
     mb((void**)&s->acts.h1, 2 * M * H);
     mb((void**)&s->acts.x3, 4 * M * H);

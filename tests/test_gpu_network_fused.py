@@ -37,3 +37,26 @@ def test_fused_kernels_agree_with_the_layer_by_layer_engine(B):
             a, b = g1[off: off + n].astype(np.float64), g0[off: off + n].astype(np.float64)
             off += n
             assert np.linalg.norm(a - b) <= 5e-3 * np.linalg.norm(b), (o, i, n)
+
+
+def _batch(B, seed):
+    rng = np.random.default_rng(seed)
+    mask = (rng.uniform(size=(B, 8)) < 0.5).astype(np.float32)
+    mask[:, 0] = 1.0
+    return (rng.uniform(-1.0, 1.0, (B, 8, 7)).astype(np.float32), mask, rng.normal(size=(B, 8, 4)).astype(np.float32))
+
+
+@pytest.mark.parametrize("max_batch", [1601, 2048, 4096])
+def test_smaller_batches_of_a_large_network(max_batch):
+    """Batches well below the network's largest (a training minibatch beside a held-out set) need more
+    partial gradients than a full one: the same bits as in a network made for the batch."""
+    import paper_2205_06557_gb300 as od
+
+    big = od.Surrogate(max_batch=max_batch, seed=3)
+    for B in (1, 16, 17, 25, 128, 1600, min(max_batch, 2048), max_batch, 128):
+        args = _batch(B, B)
+        one = od.Surrogate(max_batch=B, seed=3)
+        (l0, g0), (l1, g1) = one.gradients(*args), big.gradients(*args)
+        assert l0 == l1 and np.array_equal(g0, g1), B
+        one.close()
+    big.close()
