@@ -120,6 +120,10 @@ int batch_build(od_batch* b)
     if (!fk.empty())
         OD_BCK(b, cudaMemcpyAsync(b->d_tasks_f, fk.data(), sizeof(int2) * fk.size(), cudaMemcpyHostToDevice, b->stream));
     b->grid = (int)std::max(1ll, std::min<long long>(ctas, b->T));
+    // the counters grow by this plan's numbers of tasks and CTAs from step to step: a new plan starts
+    // them again (a reported error stays)
+    OD_BCK(b, cudaMemsetAsync(b->d_bc, 0, offsetof(BatchCtrl, err), b->stream));
+    OD_BCK(b, cudaMemsetAsync(b->d_done, 0, sizeof(unsigned long long) * 3 * R, b->stream));
     OD_BCK(b, cudaStreamSynchronize(b->stream));
     b->graph_ok = false;
     return OD_OK;
@@ -220,7 +224,6 @@ int od_create_batch(const od_params* ps, int32_t R, od_batch** out)
         b->err = "batch allocation failed";
         return fail_out(OD_ENOMEM);
     }
-    cudaMemsetAsync(b->d_done, 0, sizeof(unsigned long long) * 3 * R, b->stream);
     cudaMemsetAsync(b->d_bc, 0, sizeof(BatchCtrl), b->stream);
     rc = batch_build(b);
     if (rc) return fail_out(rc);

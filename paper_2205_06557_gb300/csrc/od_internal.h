@@ -201,7 +201,7 @@ struct RunDesc {
 
 // Device control block of a batched launch.
 struct BatchCtrl {
-    unsigned long long step;       // batched steps completed
+    unsigned long long step;       // batched steps completed with the present plan
     unsigned long long task_next;  // monotone task dispenser
     unsigned exit_count;
     int err;

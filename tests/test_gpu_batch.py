@@ -99,3 +99,23 @@ def test_batch_member_cannot_be_stepped_alone():
         od.od_step(batch.runs[0].h, 1)
     assert ei.value.code == -1
     batch.close()
+
+
+def test_new_plans_between_steps_keep_results():
+    """another plan after steps were taken (fewer and more tasks and CTAs, and the tuner's): the next steps
+    run all of its tasks"""
+    ps = _params()
+    batch = od.Batch(ps)
+    singles = [od.Run(p) for p in ps]
+    batch.step(5)
+    for tpt, chunk in ((8, 0), (2, 256), (4, 4096)):
+        od.od_batch_set_config(batch.b, tpt, chunk)
+        batch.step(5)
+    batch.tune(reps=1)
+    batch.step(5)
+    for s in singles:
+        s.step(25)
+    for r, s in zip(batch.runs, singles):
+        _compare(r, s, 25)
+        assert r.counters()[13] == 25
+    batch.close()
