@@ -357,6 +357,11 @@ int od_gemm_bf16(const uint16_t* A, const uint16_t* B, const float* bias, float*
  * 256 ions. */
 int od_selftest_wait_timeout(od_handle* h, int64_t polls);
 
+/* Self-test of the rule by which od_get_ions and od_set_ions let a kernel use a host array in
+ * place: 1 if these bytes are 8-byte aligned and lie in one page-locked allocation or
+ * registration, else 0 (such arrays go through the library's own staging).  Host only. */
+int od_selftest_host_direct(const void* p, int64_t bytes);
+
 /* Text of the last error on h, or of the last failed call without a handle (od_create,
  * od_pair_accel_static) when h is NULL. */
 const char* od_last_error(const od_handle* h);

@@ -109,6 +109,7 @@ def lib():
         L.od_set_force_config.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int]
         L.od_get_force_config.argtypes = [vp, vp, vp, vp, vp]
         L.od_selftest_wait_timeout.argtypes = [vp, i64]
+        L.od_selftest_host_direct.argtypes = [vp, i64]
         L.od_create_batch.argtypes = [vp, i32, P(vp)]
         L.od_batch_step.argtypes = [vp, i64]
         L.od_batch_run.argtypes = [vp, i32]
@@ -150,7 +151,8 @@ def lib():
         for name in ("od_sur_create", "od_sur_num_params", "od_sur_get_params", "od_sur_set_params", "od_sur_forward",
                      "od_sur_gradients", "od_sur_train_step"):
             getattr(L, name).restype = ctypes.c_int
-        for name in ("od_tune", "od_set_force_config", "od_get_force_config", "od_selftest_wait_timeout"):
+        for name in ("od_tune", "od_set_force_config", "od_get_force_config", "od_selftest_wait_timeout",
+                     "od_selftest_host_direct"):
             getattr(L, name).restype = ctypes.c_int
         for name in ("od_create", "od_step", "od_dust_state", "od_dust_terms", "od_series", "od_counters",
                      "od_dust_now", "od_set_ions", "od_info", "od_set_profiling", "od_kernel_times"):
@@ -364,6 +366,11 @@ def od_last_error(h=None):
 def od_selftest_wait_timeout(h, polls=2000):
     """return code of the bounded-wait self-test (OD_ETIMEOUT = -6 expected)"""
     return lib().od_selftest_wait_timeout(h, int(polls))
+
+
+def od_selftest_host_direct(address, nbytes):
+    """whether a kernel may use these bytes of host memory in place (one page-locked range)"""
+    return bool(lib().od_selftest_host_direct(ctypes.c_void_p(address), int(nbytes)))
 
 
 # (threads per block, targets per thread, kind) of each pair-kernel variant: kind 0 the

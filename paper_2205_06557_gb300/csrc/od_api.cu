@@ -5,6 +5,8 @@
 // plans the pair-kernel partition, allocates device memory and places the initial
 // ions; od_step replays a captured graph of one step (or launches its kernels
 // directly in profiling mode).
+#include <cuda.h>  // the driver's types (no link to libcuda)
+
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
@@ -732,22 +734,37 @@ int ensure_io(od_handle* h)
     return OD_OK;
 }
 
-// whether a kernel can address these bytes of host memory (page-locked or registered from the
-// first to the last, 8-byte aligned), and their address on the GPU
+// whether a kernel can address these bytes of host memory (8-byte aligned, all in one page-locked
+// allocation or registration), and their address on the GPU.  The two ends alone do not show it:
+// they may lie in two registrations with pageable memory between.  The range comes from the
+// driver's cuPointerGetAttribute, fetched through the runtime (no link to libcuda).
 bool host_direct(const void* p, size_t bytes, void** dev)
 {
     if (((uintptr_t)p & 7) || bytes < 8) return false;
-    cudaPointerAttributes at[2]{};
-    const char* const ends[2] = {(const char*)p, (const char*)p + bytes - 1};
-    for (int k = 0; k < 2; ++k)
-        if (cudaPointerGetAttributes(&at[k], ends[k]) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        } else if (at[k].type != cudaMemoryTypeHost || !at[k].devicePointer) {
-            return false;
-        }
-    if ((char*)at[1].devicePointer - (char*)at[0].devicePointer != ends[1] - ends[0]) return false;
-    *dev = at[0].devicePointer;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (at.type != cudaMemoryTypeHost || !at.devicePointer) return false;
+    typedef CUresult (*GetAttribute)(void*, CUpointer_attribute, CUdeviceptr);
+    static const GetAttribute get = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 12000, cudaEnableDefault, &q) ==
+                            cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        cudaGetLastError();
+        return ok ? (GetAttribute)fn : nullptr;
+    }();
+    const CUdeviceptr d = (CUdeviceptr)at.devicePointer;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    if (!get || get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, d) != CUDA_SUCCESS ||
+        get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, d) != CUDA_SUCCESS || d < start || bytes > size ||
+        d - start > size - bytes)
+        return false;
+    *dev = at.devicePointer;
     return true;
 }
 
@@ -1276,6 +1293,12 @@ int od_selftest_wait_timeout(od_handle* h, int64_t polls)
     OD_CK(h, cudaStreamSynchronize(h->stream));
     h->graph_ok = false;
     return read_error_word(h);
+}
+
+int od_selftest_host_direct(const void* p, int64_t bytes)
+{
+    void* dev = nullptr;
+    return p && bytes > 0 && host_direct(p, (size_t)bytes, &dev) ? 1 : 0;
 }
 
 int od_num_dust(od_handle* h) { return h ? h->P.D : fail(h, OD_EINVAL, "bad handle"); }

@@ -159,3 +159,34 @@ def test_step_graph_lengths_give_the_same_bits():
             assert np.array_equal(a, b)
     for r in runs:
         r.close()
+
+
+def test_host_arrays_used_in_place_lie_in_one_page_locked_range():
+    """an array whose two ends are page-locked by two registrations, with pageable memory between, is
+    not handed to a kernel; pieces of one registration or allocation are (host side only)"""
+    import mmap
+
+    import torch
+
+    page, rt = 65536, torch.cuda.cudart()
+    buf = mmap.mmap(-1, 4 * page)
+    raw = np.frombuffer(buf, dtype=np.uint8)
+    raw[:] = 1
+    p0 = -(-raw.ctypes.data // page) * page  # two whole pages with one between
+    assert not od.od_selftest_host_direct(p0, 3 * page)
+    for p in (p0, p0 + 2 * page):
+        assert int(rt.cudaHostRegister(p, page, 0)) == 0
+    try:
+        for p in (p0, p0 + 2 * page):
+            assert od.od_selftest_host_direct(p, page)
+            assert od.od_selftest_host_direct(p + 8, page - 8)
+            assert not od.od_selftest_host_direct(p + 4, 64)
+        assert not od.od_selftest_host_direct(p0, 3 * page)
+        assert not od.od_selftest_host_direct(p0 + 8, 2 * page)
+        assert not od.od_selftest_host_direct(p0, page + 8)
+    finally:
+        for p in (p0, p0 + 2 * page):
+            rt.cudaHostUnregister(p)
+    t = torch.zeros(5000, dtype=torch.float64, pin_memory=True)
+    assert od.od_selftest_host_direct(t.data_ptr(), 40000) and od.od_selftest_host_direct(t.data_ptr() + 800, 39200)
+    assert not od.od_selftest_host_direct(t.data_ptr(), 1 << 40)
