@@ -389,9 +389,9 @@ const char* od_last_error(const od_handle* h);
  * allocating library routine is called.  The first call on a device (and the first after
  * its context changes, e.g. after cudaDeviceReset) looks up the array's device address
  * with that device current; make that first call before any stream capture.  Every call
- * shares the one array and leaves its contents behind: the bound word carries the number of
- * its call (a captured call clears it), everything else it reads is written by the same call
- * first.
+ * shares the one array and leaves its contents behind: the bound word and the cells' lists
+ * carry the number of their call (a captured call, which is replayed with its number, clears
+ * them first), everything else it reads is written by the same call first.
  * Calls whose work overlaps on the GPU (different streams, or different host threads on
  * one device) race on the array and give wrong results: serialise them. */
 #define OD_STATIC_MAX_IONS 32768

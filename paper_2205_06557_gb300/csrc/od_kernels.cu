@@ -1121,13 +1121,16 @@ extern "C" int od_pair_accel_static(const double* x, int64_t n, double lambda_De
     unsigned long long* head = (unsigned long long*)(base + kOffHead);
     int* next = (int*)(base + kOffNext);
     unsigned long long* bound = (unsigned long long*)(base + kOffBound);
-    // epoch 1 follows the wrap (the older word would be larger); a captured call is replayed
-    // with its epoch, so there the word is cleared
+    // epoch 1 follows the wrap (the older words would be larger, or tagged the same); a captured call
+    // is replayed with its epoch, so its nodes clear the bound word and the buckets first
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool asked = cudaStreamIsCapturing(s, &cap) == cudaSuccess;
     if (!asked) cudaGetLastError();
-    const bool capturing = !asked || cap != cudaStreamCaptureStatusNone;
-    cudaError_t e = epoch == 1 || capturing ? cudaMemsetAsync(bound, 0, sizeof(*bound), s) : cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if (epoch == 1 || !asked || cap != cudaStreamCaptureStatusNone) {
+        e = cudaMemsetAsync(bound, 0, sizeof(*bound), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(head, 0, sizeof(*head) * kStaticBuckets, s);
+    }
     if (e == cudaSuccess) {
         // small blocks spread the FP64 work (slow on this GPU) over the SMs
         k_static_bound<<<(int)((n + 127) / 128), 128, 0, s>>>(x, (int)n, ls_inv, epoch, bound);
