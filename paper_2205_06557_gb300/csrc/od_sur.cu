@@ -307,6 +307,7 @@ struct od_sur {
     float *h1 = nullptr, *h2 = nullptr, *c = nullptr, *h3 = nullptr, *h4 = nullptr, *yp = nullptr, *dy = nullptr,
           *dx3 = nullptr, *da = nullptr;
     cudaStream_t stream = nullptr;
+    cudaEvent_t ev_in = nullptr;  // after the copies of a batch's host arrays, in a call that reads no result
     long long adam_t = 0;
     int engine = OD_GEMM_TCGEN05;
     std::string err;
@@ -377,6 +378,7 @@ void free_sur(od_sur* s)
                     s->tA, s->tB, s->h1, s->h2, s->c, s->h3, s->h4, s->yp, s->dy, s->dx3, s->da};
     for (void* p : bufs) cudaFree(p);
     cudaFreeHost(s->h_out);
+    if (s->ev_in) cudaEventDestroy(s->ev_in);
 }
 
 // buffers of the layer-by-layer engine
@@ -462,8 +464,9 @@ int backward_layers(od_sur* s, int Bn, float inv_count)
     return cudaGetLastError() == cudaSuccess ? OD_OK : sfail(s, OD_ECUDA, "backward launch failed");
 }
 
-// the batch's arrays as they come; the layer-by-layer engine takes an even number of samples,
-// the last of an odd batch absent and zero
+// The batch's arrays as they come; the layer-by-layer engine takes an even number of samples,
+// the last of an odd batch absent and zero.  Copies of page-locked arrays are still under way on
+// return: a call ends with read_out, or waits for them itself.
 int upload_batch(od_sur* s, const float* x, const float* mask, const float* tgt, int Bn)
 {
     const size_t M = (size_t)Bn * G;
@@ -476,6 +479,13 @@ int upload_batch(od_sur* s, const float* x, const float* mask, const float* tgt,
         SCK(s, cudaMemsetAsync(s->tgt + M * OUTR, 0, sizeof(float) * G * OUTR, s->stream));
     }
     return OD_OK;
+}
+
+// the end of a call that failed: the host arrays are the caller's again
+int give_back(od_sur* s, int rc)
+{
+    cudaStreamSynchronize(s->stream);
+    return rc;
 }
 
 mlp::FusedArgs fused_args(od_sur* s, int Bn)
@@ -588,7 +598,8 @@ int od_sur_create(int max_batch, uint64_t seed, void* stream, od_sur** out)
     mb((void**)&s->acts.dz2, 2 * M * H);
     mb((void**)&s->acts.dz1, 2 * M * H);
     mb((void**)&s->d_out, sizeof(SurOut));
-    ok = ok && cudaMallocHost((void**)&s->h_out, sizeof(SurOut)) == cudaSuccess;
+    ok = ok && cudaMallocHost((void**)&s->h_out, sizeof(SurOut)) == cudaSuccess &&
+         cudaEventCreateWithFlags(&s->ev_in, cudaEventDisableTiming) == cudaSuccess;
     if (ok) {
         std::vector<float> p(mlp::N_PARAMS, 0.f);
         long long wo = 0;
@@ -674,8 +685,7 @@ int od_sur_forward(od_sur* s, const float* x, const float* mask, int Bn, float* 
 {
     if (!s || !x || !mask || !y || Bn < 1 || Bn > s->maxB) return sfail(s, OD_EINVAL, "bad forward arguments");
     int rc = upload_batch(s, x, mask, nullptr, Bn);
-    if (rc) return rc;
-    if ((rc = run_forward(s, Bn))) return rc;
+    if (rc || (rc = run_forward(s, Bn))) return give_back(s, rc);
     SCK(s, cudaMemcpyAsync(y, s->y, sizeof(float) * Bn * G * OUTR, cudaMemcpyDeviceToHost, s->stream));
     return read_out(s);
 }
@@ -685,11 +695,15 @@ int od_sur_gradients(od_sur* s, const float* x, const float* mask, const float* 
 {
     if (!s || !x || !mask || !tgt || Bn < 1 || Bn > s->maxB) return sfail(s, OD_EINVAL, "bad gradient arguments");
     int rc = upload_batch(s, x, mask, tgt, Bn);
-    if (rc) return rc;
-    if ((rc = run_gradients(s, Bn, mask))) return rc;
+    const bool reads = grads || loss;  // else the call waits for the copies only, not for the kernels
+    if (!rc && !reads) SCK(s, cudaEventRecord(s->ev_in, s->stream));
+    if (rc || (rc = run_gradients(s, Bn, mask))) return give_back(s, rc);
     if (grads)
         SCK(s, cudaMemcpyAsync(grads, s->g, sizeof(float) * mlp::N_PARAMS, cudaMemcpyDeviceToHost, s->stream));
-    if (!grads && !loss) return OD_OK;
+    if (!reads) {
+        SCK(s, cudaEventSynchronize(s->ev_in));
+        return OD_OK;
+    }
     if ((rc = read_out(s))) return rc;
     if (loss) *loss = s->h_out->loss;
     return OD_OK;

@@ -60,3 +60,30 @@ def test_smaller_batches_of_a_large_network(max_batch):
         assert l0 == l1 and np.array_equal(g0, g1), B
         one.close()
     big.close()
+
+
+def test_train_step_without_a_loss_has_read_its_inputs():
+    """The caller's arrays are its own again when the call returns, page-locked ones too: they are
+    overwritten at once, while the stream is still busy with work queued before the call."""
+    import torch
+
+    import paper_2205_06557_gb300 as od
+
+    B = 512
+    host = [torch.from_numpy(v).pin_memory() for v in _batch(B, 5)]
+    stream = torch.cuda.Stream()
+    params = []
+    for overwrite in (False, True):
+        net = od.Surrogate(max_batch=B, seed=1, stream=stream.cuda_stream)
+        arr = [h.clone().pin_memory() for h in host]
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(20_000_000)  # ~10 ms
+        vp = od.ctypes.c_void_p
+        rc = od.lib().od_sur_train_step(net.h, *(vp(t.data_ptr()) for t in arr), B, od.ctypes.c_float(1e-3), None)
+        if overwrite:
+            for t in arr:
+                t.fill_(0.25)
+        assert rc == 0
+        params.append(net.get_params())
+        net.close()
+    assert np.array_equal(params[0], params[1])
