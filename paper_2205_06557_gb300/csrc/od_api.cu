@@ -1165,8 +1165,8 @@ int od_dust_now(od_handle* h, double* q, double* f_orbit)
 int64_t od_get_ions(od_handle* h, double* x, double* v, double* a, uint64_t* id, int64_t cap)
 {
     if (!h) return fail(h, OD_EINVAL, "bad handle");
-    long long N = h->P.N;  // ions alive: varies under the flux rule
-    if (h->P.flags & OD_F_FLUX_INJECT) {
+    long long N = h->P.N;  // ions alive
+    if ((h->P.flags & OD_F_FLUX_INJECT) || !h->plan_is_live) {
         const int rc = read_ctrl(h);
         if (rc) return rc;
         N = h->h_area->ctrl.n_cur;
@@ -1223,6 +1223,7 @@ int od_set_ions(od_handle* h, const double* x, const double* v, const double* a,
         return rc;
     }
     if (h->P.N != n_plan_old) h->graph_ok = false;
+    h->plan_is_live = true;
     // given accelerations were converted on the device above (the positions and their
     // close-pair lists are refreshed); otherwise evaluate them
     if (a) OD_LK(h, launch_fpos(h->P, h->B, buf, h->stream));

@@ -42,6 +42,8 @@ struct od_handle {
     cudaGraph_t graph_k = nullptr;  // STEP_GRAPH_K steps in one graph (long od_step calls)
     cudaGraphExec_t gexec_k = nullptr;
     bool graph_k_ok = false;
+    bool plan_is_live = true;  // the planned ion count is the number alive, except under the flux rule and in a
+                               // run loaded without ions (planned for the creation's)
     long long cap = 0;       // ion capacity
     long long npad_cap = 0;  // fpos capacity
     long long part_cap = 0;  // partial-sum capacity (float4)

@@ -222,6 +222,7 @@ int od_load(const char* path, void* cuda_stream, od_handle** out)
     h->prm.n_ions = hd.n_ions;
     if (hd.r_cut > 0.0 && (rc = od_set_cutoff(h, hd.r_cut, hd.r_switch))) return done(rc);
     h->host_step = hd.step;
+    h->plan_is_live = N > 0;
     const int buf = (int)(hd.step & 1);
     if (N > 0) {
         std::vector<double> tmp(3 * (size_t)N);

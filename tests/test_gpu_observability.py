@@ -190,3 +190,22 @@ def test_host_arrays_used_in_place_lie_in_one_page_locked_range():
     t = torch.zeros(5000, dtype=torch.float64, pin_memory=True)
     assert od.od_selftest_host_direct(t.data_ptr(), 40000) and od.od_selftest_host_direct(t.data_ptr() + 800, 39200)
     assert not od.od_selftest_host_direct(t.data_ptr(), 1 << 40)
+
+
+def test_checkpoint_without_ions(tmp_path):
+    """a state without ions stays one across a checkpoint: the reads give no ions (the plan of the
+    restored run is still the creation's), and a state put in afterwards is read back whole"""
+    p = W.tiny()
+    a = od.Run(p)
+    a.set_ions(np.zeros((0, 3)), np.zeros((0, 3)), np.zeros(0, dtype=np.uint64), next_id=7)
+    assert len(a.get_ions()[0]) == 0
+    path = str(tmp_path / "empty.ckpt")
+    a.save(path)
+    b = od.Run.load(path)
+    assert all(len(t) == 0 for t in b.get_ions()) and b.counters()[14] == 0
+    x, v, ids = W.random_ions(100, p["R"], p["H"], seed=3, dust=p["dust"])
+    b.set_ions(x, v, ids, next_id=100)
+    xb, vb, _, ib = b.get_ions()
+    assert np.array_equal(xb, x) and np.array_equal(vb, v) and np.array_equal(ib, ids)
+    a.close()
+    b.close()
