@@ -209,3 +209,23 @@ def test_checkpoint_without_ions(tmp_path):
     assert np.array_equal(xb, x) and np.array_equal(vb, v) and np.array_equal(ib, ids)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("grains", [0, 1, 3])
+def test_series_of_any_length_are_parts_of_the_whole(grains):
+    """ranges below and above the length from which they are copied whole, ragged ones, records or events
+    alone: the parts of the whole series"""
+    p = W.tiny()
+    p["dust"] = [dict(x=0.0, y=0.0, z=6e-5 * (k - 1), a=1e-5, q0=-2e-15) for k in range(grains)]
+    r = od.Run(p)
+    r.step(300)
+    rec, ev = (np.concatenate(v) for v in zip(*(r.series(s, 50) for s in range(1, 301, 50))))
+    assert rec.shape[:2] == (300, grains) and ev.shape[0] == 300 and ev.any()
+    for first, count in ((1, 300), (1, 256), (2, 257), (3, 129), (17, 128), (300, 1), (5, 0)):
+        a, b = r.series(first, count)
+        assert np.array_equal(a, rec[first - 1: first - 1 + count]) and np.array_equal(b, ev[first - 1: first - 1 + count])
+    for count in (200, 290):
+        a, b = np.zeros_like(rec[:count]), np.zeros_like(ev[:count])
+        assert od.lib().od_series(r.h, 1, count, a.ctypes.data, None) == 0 and np.array_equal(a, rec[:count])
+        assert od.lib().od_series(r.h, 1, count, None, b.ctypes.data) == 0 and np.array_equal(b, ev[:count])
+    r.close()
