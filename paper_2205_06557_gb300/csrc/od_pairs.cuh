@@ -402,11 +402,9 @@ struct WarpStage {
     f32x2 x[64], y[64], z[64];
 };
 
-// Sources pa (ion `lane` of the group) and pb (ion 32 + lane).  BOTH: the sources' sums go to b
-// (x, y, z of ion `lane`, then of ion 32 + lane) with the target-side sign; otherwise (a group
-// of the targets' own tile: each ordered pair met once) only the targets' sums are made, and
-// a self pair (d = 0) adds nothing.  CUT: the switched coefficient.
-template <int IPT, bool CUT, bool BOTH>
+// Sources pa (ion `lane` of the group) and pb (ion 32 + lane).  The sources' sums go to b (x, y, z of
+// ion `lane`, then of ion 32 + lane) with the target-side sign.  CUT: the switched coefficient.
+template <int IPT, bool CUT>
 __device__ __forceinline__ void sym2_group(float4 pa, float4 pb, const float (&xi)[IPT], const float (&yi)[IPT],
                                            const float (&zi)[IPT], f32x2 (&ax)[IPT], f32x2 (&ay)[IPT],
                                            f32x2 (&az)[IPT], float (&b)[6], WarpStage& S, float s0, float w_inv)
@@ -426,26 +424,20 @@ __device__ __forceinline__ void sym2_group(float4 pa, float4 pb, const float (&x
             const f32x2 dx = sub2(xj, pk2(xi[k], xi[k])), dy = sub2(yj, pk2(yi[k], yi[k])),
                         dz = sub2(zj, pk2(zi[k], zi[k]));
             const f32x2 c3 = CUT ? pair_c3x2_cut(dx, dy, dz, s0, w_inv) : pair_c3x2(dx, dy, dz);
-            if (BOTH) {
-                bx = fma2(c3, dx, bx);
-                by = fma2(c3, dy, by);
-                bz = fma2(c3, dz, bz);
-            }
+            bx = fma2(c3, dx, bx);
+            by = fma2(c3, dy, by);
+            bz = fma2(c3, dz, bz);
             ax[k] = fma2(c3, dx, ax[k]);
             ay[k] = fma2(c3, dy, ay[k]);
             az[k] = fma2(c3, dz, az[k]);
         }
-        if (BOTH) {
-            bx = __shfl_sync(0xffffffffu, bx, src);
-            by = __shfl_sync(0xffffffffu, by, src);
-            bz = __shfl_sync(0xffffffffu, bz, src);
-        }
+        bx = __shfl_sync(0xffffffffu, bx, src);
+        by = __shfl_sync(0xffffffffu, by, src);
+        bz = __shfl_sync(0xffffffffu, bz, src);
     }
-    if (BOTH) {
-        upk2(bx, b[0], b[3]);
-        upk2(by, b[1], b[4]);
-        upk2(bz, b[2], b[5]);
-    }
+    upk2(bx, b[0], b[3]);
+    upk2(by, b[1], b[4]);
+    upk2(bz, b[2], b[5]);
 }
 
 // Sources per combine step of a CTA of NW warps and tiles of TI ions: the warps meet at two
@@ -499,8 +491,8 @@ __device__ __forceinline__ void sym2_unit(const float4* __restrict__ fpos, const
             for (int q = 0; q < SUB / SYM_GRP; ++q) {
                 const int jq = q * SYM_GRP + lane;
                 float b[6];
-                sym2_group<IPT, CUT, true>(__ldg(fpos + jb + jq), __ldg(fpos + jb + jq + 32), xi, yi, zi, ax2, ay2,
-                                           az2, b, S.stage[w], F.cut_s0, F.cut_inv_w);
+                sym2_group<IPT, CUT>(__ldg(fpos + jb + jq), __ldg(fpos + jb + jq + 32), xi, yi, zi, ax2, ay2,
+                                     az2, b, S.stage[w], F.cut_s0, F.cut_inv_w);
                 if (NW == 1) {
                     fixed_add3(F.psum, F.psum_ld, jb + jq, -b[0], -b[1], -b[2], F.qscale, F.err);
                     fixed_add3(F.psum, F.psum_ld, jb + jq + 32, -b[3], -b[4], -b[5], F.qscale, F.err);
