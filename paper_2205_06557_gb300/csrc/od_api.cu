@@ -1234,16 +1234,20 @@ int od_set_ions(od_handle* h, const double* x, const double* v, const double* a,
     // the step graph holds the plan by value and the plan is a function of the planned
     // ion count: keep it when that is unchanged
     const int n_plan_old = h->P.N;
-    if ((rc = replan(h, plan_n(h, n)))) {
+    rc = replan(h, plan_n(h, n));
+    if (!rc) {
+        if (h->P.N != n_plan_old) h->graph_ok = false;
+        h->plan_is_live = true;
+        // given accelerations were converted on the device above (the positions and their
+        // close-pair lists are refreshed); otherwise evaluate them
+        if (!a) rc = force_eval(h);
+        else if (const int e = launch_fpos(h->P, h->B, buf, h->stream))
+            rc = cuda_fail(h, (cudaError_t)e, "launch_fpos");
+    }
+    if (rc) {
         cudaStreamSynchronize(h->stream);  // the host arrays are the caller's again
         return rc;
     }
-    if (h->P.N != n_plan_old) h->graph_ok = false;
-    h->plan_is_live = true;
-    // given accelerations were converted on the device above (the positions and their
-    // close-pair lists are refreshed); otherwise evaluate them
-    if (a) OD_LK(h, launch_fpos(h->P, h->B, buf, h->stream));
-    else if ((rc = force_eval(h))) return rc;
     return read_error_word(h);
 }
 
