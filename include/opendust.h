@@ -285,9 +285,10 @@ int od_oml_charge(const od_params* p, double radius, double* Q);
  *                     0}, where chunk 0 means symmetric tile pairs of 128 x targets-per-
  *                     thread ions (each unordered pair once, packed FP32 pairs, one partial
  *                     slot per tile for every ion); ms[12] (host, may be NULL) gets the
- *                     average ms per launch, [ipt index][chunk index]; keeps the fastest and
- *                     recomputes the accelerations with it; positions, velocities and
- *                     grain state are not changed
+ *                     average ms per launch, [ipt index][chunk index]; keeps the fastest (of
+ *                     two numbers of targets per thread at one chunk that time within 1%,
+ *                     for 8 targets 2%, the larger) and recomputes the accelerations with
+ *                     it; positions, velocities and grain state are not changed
  *   od_batch_set_config applies a known choice (targets per thread 2, 4 or 8; chunk 0
  *                     or >= 256); od_destroy_batch
  *                     frees everything

@@ -12,7 +12,8 @@
 // tiles; every task waited for was handed out earlier to a CTA that is running, so the waits
 // end (and each is bounded anyway: it gives up after spin_limit polls and sets an error).
 // The counters only grow (target = (batch step + 1) x tasks of the kind), so nothing
-// is reset between launches; the last CTA to leave advances the batch step.
+// is reset between launches; the last CTA to leave advances the batch step.  A new plan
+// (other numbers of tasks and CTAs) starts them again.
 // What bounds it: the latency of a step's chain (scan, pair units, kick) and, between, the FP32 pipe
 // for the pair units and the FP64 pipe for the rest, which is why the two are mixed.  48 runs of
 // 2,171 ions (tile pairs of 256 ions), per step: 223 us with the ion terms and grain sums

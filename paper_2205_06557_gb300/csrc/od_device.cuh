@@ -108,8 +108,7 @@ __device__ __forceinline__ void inj_angle(int face, uint4 A, double& s, double& 
 }
 
 // axial speed through a cap: the tabulated inverse CDF brackets the root and gives the
-// starting point, Newton polishes it to ~1e-13 (a few iterations instead of a bisection
-// from the whole range)
+// starting point, from which most samples need one of invert_flux's steps
 __device__ __forceinline__ double inj_axial(const Phys& P, int face, uint4 A)
 {
     const double U = unif(A.w);

@@ -114,7 +114,7 @@ struct Phys {
     double e_over_kTe;
     double inv4pieps0;
     // App. B inverse flux CDFs tabulated at U = k / VTAB_K (bottom face, then top face):
-    // starting points and brackets for the Newton polish of every injected axial speed; then
+    // starting points and brackets of every injected axial speed's inversion; then
     // Phi(-u / sig), phi(-u / sig) and 1 / sig
     const double* vtab;
     double gmax_b, gmax_t;  // flux integrals G(v_max) and G_top(v_min) the CDFs are normalised by
